@@ -17,6 +17,7 @@
 #include <stdint.h>
 
 #include "hg_internal.cuh"
+#include "hg_pair64.cuh"
 
 namespace hg {
 namespace {
@@ -60,6 +61,8 @@ struct Mixed {
         float n[I];   // noise scale (positive terms, plain sums of kFold-term chunks)
     };
     typedef float Eps;
+
+    __device__ static Eps soften(double eps2) { return (Eps)eps2; }
 
     __device__ static void load_i(const Records &rec, int r, IData &d)
     {
@@ -358,49 +361,38 @@ struct Mixed {
 };
 
 // ------------------------------------------------------------------------
-// FP64 throughout.
+// FP64 path: FP64 records and sums, the pair law in block fixed point on the
+// integer pipes (hg_pair64.cuh).
+// With the whole pair law in FP64 instructions the kernel kept the FP64 unit 91 %
+// busy; m = N = 32768 took 99.5 ms, now 37.6 ms (the nine differences hold the FP64
+// unit 44 % of the time, the ALU pipe is 66 % busy).  Errors against 64-bit
+// arithmetic stayed below those of the FP64 instructions.
 // ------------------------------------------------------------------------
 struct F64 {
     static constexpr int TJ = kTJF64;
-    static constexpr int I = kIF64;
-    static constexpr int kMinBlocks = 2;
+    static constexpr int I = 1;
+    static constexpr int kMinBlocks = 3;
     static constexpr int kVariant = 0;
     static constexpr uint32_t kStageBytes = TJ * 80;
-    struct IData {
-        double x, y, z, vx, vy, vz, ax, ay, az;
-    };
     struct ITile {
-        IData d[I];
+        p64::Body d[I];
     };
-    struct Acc {
-        double s[I][9];
-    };
-    typedef double Eps;
+    typedef p64::Sums Acc;
+    typedef p64::Soft Eps;
 
-    __device__ static void load_i(const Records &rec, int i, IData &d)
+    __device__ static Eps soften(double eps2) { return p64::soft(eps2); }
+
+    __device__ static void zero(Acc &a) { p64::clear(a); }
+
+    __device__ static void load(const Records &rec, const int (&ids)[I], ITile &t)
     {
+        const int i = ids[0];
         const double2 q0 = __ldcg(static_cast<const double2 *>(rec.p[0]) + i);
         const double2 q1 = __ldcg(static_cast<const double2 *>(rec.p[1]) + i);
         const double2 q2 = __ldcg(static_cast<const double2 *>(rec.p[2]) + i);
         const double2 q3 = __ldcg(static_cast<const double2 *>(rec.p[3]) + i);
         const double2 q4 = __ldcg(static_cast<const double2 *>(rec.p[4]) + i);
-        d.x = q0.x; d.y = q0.y; d.z = q1.x;
-        d.vx = q2.x; d.vy = q2.y; d.vz = q3.x;
-        d.ax = q3.y; d.ay = q4.x; d.az = q4.y;
-    }
-
-    __device__ static void zero(Acc &a)
-    {
-#pragma unroll
-        for (int k = 0; k < I; ++k)
-#pragma unroll
-            for (int c = 0; c < 9; ++c) a.s[k][c] = 0.0;
-    }
-
-    __device__ static void load(const Records &rec, const int (&ids)[I], ITile &t)
-    {
-#pragma unroll
-        for (int k = 0; k < I; ++k) load_i(rec, ids[k], t.d[k]);
+        t.d[0] = p64::Body{q0.x, q0.y, q1.x, q2.x, q2.y, q3.x, q3.y, q4.x, q4.y};
     }
 
     __device__ static void issue(const Records &rec, int64_t tile, unsigned char *dst, uint64_t *bar,
@@ -414,49 +406,16 @@ struct F64 {
     }
 
     template <bool GUARD>
-    __device__ __forceinline__ static void pair(const IData &d, const double2 q0, const double2 q1,
-                                                const double2 q2, const double2 q3, const double2 q4,
-                                                const double eps2, double (&s)[9])
-    {
-        const double dx = q0.x - d.x, dy = q0.y - d.y, dz = q1.x - d.z;
-        const double dvx = q2.x - d.vx, dvy = q2.y - d.vy, dvz = q3.x - d.vz;
-        const double dax = q3.y - d.ax, day = q4.x - d.ay, daz = q4.y - d.az;
-        const double r2 = fma(dz, dz, fma(dy, dy, fma(dx, dx, eps2)));
-        double rinv = rsqrt(r2);
-        if (GUARD) rinv = (r2 > 0.0) ? rinv : 0.0;
-        const double rinv2 = rinv * rinv;
-        const double q = q1.y * rinv * rinv2;
-        const double rv = fma(dz, dvz, fma(dy, dvy, dx * dvx));
-        const double v2ra = fma(dz, daz, fma(dy, day, fma(dx, dax, fma(dvz, dvz, fma(dvy, dvy, dvx * dvx)))));
-        const double alpha = rv * rinv2;
-        const double beta = fma(alpha, alpha, v2ra * rinv2);
-        const double a3 = -3.0 * alpha;
-        const double a6 = a3 + a3, b3 = -3.0 * beta;
-        const double wx = fma(a3, dx, dvx), wy = fma(a3, dy, dvy), wz = fma(a3, dz, dvz);
-        s[0] = fma(q, dx, s[0]);
-        s[1] = fma(q, dy, s[1]);
-        s[2] = fma(q, dz, s[2]);
-        s[3] = fma(q, wx, s[3]);
-        s[4] = fma(q, wy, s[4]);
-        s[5] = fma(q, wz, s[5]);
-        s[6] = fma(q, fma(b3, dx, fma(a6, wx, dax)), s[6]);
-        s[7] = fma(q, fma(b3, dy, fma(a6, wy, day)), s[7]);
-        s[8] = fma(q, fma(b3, dz, fma(a6, wz, daz)), s[8]);
-    }
-
-    template <bool GUARD>
     __device__ static void tile(const unsigned char *sb, int tpi, int lane_j, const ITile &iv, Acc &acc,
-                                Eps eps2, int64_t)
+                                const Eps &eps2, int64_t)
     {
         const double2 *q0 = reinterpret_cast<const double2 *>(sb);
-        const int jpt = TJ >> (__ffs(tpi) - 1);   // tpi a power of two
-#pragma unroll 2
-        for (int u = 0; u < jpt; ++u) {
-            const int jj = u * tpi + lane_j;
+#pragma unroll 1
+        for (int jj = lane_j; jj < TJ; jj += tpi) {
             const double2 a = q0[jj], b = q0[TJ + jj], c = q0[2 * TJ + jj], d = q0[3 * TJ + jj],
                           e = q0[4 * TJ + jj];
-#pragma unroll
-            for (int k = 0; k < I; ++k) pair<GUARD>(iv.d[k], a, b, c, d, e, eps2, acc.s[k]);
+            p64::pair<GUARD>(iv.d[0], a.x, a.y, b.x, b.y, c.x, c.y, d.x, d.y, e.x, e.y, eps2, acc);
+            p64::count_pair(acc);
         }
     }
 
@@ -465,10 +424,11 @@ struct F64 {
     // noise scale (out[k][9] = 0): the FP64 path needs no noise floor.
     __device__ static void epilogue(Acc &a, int tpi, int tid, double *red, double (&out)[I][kOut])
     {
+        p64::finish(a);
 #pragma unroll
         for (int k = 0; k < I; ++k) {
 #pragma unroll
-            for (int c = 0; c < 9; ++c) out[k][c] = a.s[k][c];
+            for (int c = 0; c < 9; ++c) out[k][c] = a.s[c];
             out[k][9] = 0.0;
         }
         const int wspan = tpi < 32 ? tpi : 32;
@@ -526,7 +486,7 @@ __device__ bool eval_items(const EvalArgs &args, int64_t m, const Plan &pl, unsi
     if (!batch && pl.variant != P::kVariant) return true;   // a plan for another kernel (none at present)
     const int64_t n_items = batch ? bv.item_off[bv.nc] : pl.n_items;
     const int64_t tps = batch ? *bv.tps : pl.tiles_per_split;
-    const typename P::Eps eps2 = (typename P::Eps)args.eps2;
+    const typename P::Eps eps2 = P::soften(args.eps2);
 
     for (int64_t item = blockIdx.x; item < n_items; item += gridDim.x) {
         // Decode the item: active positions [q_begin, q_end) of this i-tile's

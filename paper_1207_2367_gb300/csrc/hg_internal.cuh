@@ -74,7 +74,6 @@ constexpr int kStages = 3;
 constexpr int kTJMixed = 256;   // j-records per shared-memory tile, mixed
 constexpr int kTJF64 = 128;     // j-records per shared-memory tile, fp64
 constexpr int kIMixed = 1;      // i-particles held per thread, mixed
-constexpr int kIF64 = 1;        // i-particles held per thread, fp64
 constexpr int kMaxTPI = 64;
 constexpr double kPadCoord = 1.0e18;
 constexpr long long kWaitCycles = 4000000000LL;   // ~2 s at 2 GHz

