@@ -377,8 +377,8 @@ __global__ void __launch_bounds__(kPotThreads) k_potential_fp64(const double *xe
             sy[threadIdx.x] = xe[3 * j + 1];
             sz[threadIdx.x] = xe[3 * j + 2];
             p64::Limbs m;
-            uint32_t top = 0;
-            se[threadIdx.x] = p64::mass_limbs(mass[j], m, top);
+            uint32_t low = 0;
+            se[threadIdx.x] = p64::mass_limbs(mass[j], m, low);
             sm[threadIdx.x] = m;
         }
         __syncthreads();
@@ -392,7 +392,7 @@ __global__ void __launch_bounds__(kPotThreads) k_potential_fp64(const double *xe
             p64::fold_fp64(acc);
         }
     }
-    if (i < n) phi_part[blockIdx.y * n + i] = acc.top >= p64::kHiInf ? NAN : acc.s;
+    if (i < n) phi_part[blockIdx.y * n + i] = acc.low < 0x100000u ? NAN : acc.s;
 }
 
 // Independent clusters: phi_i sums over the other particles of i's own cluster

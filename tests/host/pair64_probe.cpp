@@ -30,8 +30,8 @@ int main()
                 hg::p64::pair<true>(b, j[0], j[1], j[2], m, j[3], j[4], j[5], j[6], j[7], j[8], soft, s);
             hg::p64::count_pair(s);
             hg::p64::Limbs ml;
-            uint32_t top = 0;
-            const int em = hg::p64::mass_limbs(m, ml, top);
+            uint32_t low = 0;
+            const int em = hg::p64::mass_limbs(m, ml, low);
             const bool self = j[0] == i[0] && j[1] == i[1] && j[2] == i[2];
             hg::p64::pair_potential(j[0] - i[0], j[1] - i[1], j[2] - i[2], ml, em, self, soft, p);
             if (k % hg::p64::kFold64 == hg::p64::kFold64 - 1) hg::p64::fold_fp64(p);
