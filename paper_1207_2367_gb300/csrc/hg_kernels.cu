@@ -352,27 +352,35 @@ __global__ void __launch_bounds__(kPotThreads) k_potential_mixed(const double *x
 }
 
 // FP64 pairs: the differences on the FP64 unit, the rest in block fixed point
-// (hg_pair64.cuh).  The j-particles' masses are split once per CTA and tile.  N =
-// 65536: 106 ms with FP64 instructions throughout (16 a pair, 64 cycles each per
-// warp), now 37 ms.
+// (hg_pair64.cuh).  Every pair is taken once: with T tiles of kPotThreads particles,
+// tile I meets tiles I .. I + T / 2 (modulo T), its own only for j > i and, for even
+// T, the opposite one only from I < T / 2; so every tile has the same work.  The
+// sums phi_part then hold each pair on one side: W = -sum_i m_i phi_i.  A block
+// (I, s) takes the tiles s, s + nsplit, ... of that range.  The j-particles' masses
+// are split once per block and tile.  N = 65536: 106 ms with FP64 instructions
+// throughout (16 a pair, 64 cycles each per warp) and every pair from both sides,
+// 37.1 ms in fixed point, now 16.9 ms; bound by the integer pipes' issue and the
+// three FP64 subtractions (192 of ~330 cycles per warp and pair).
 __global__ void __launch_bounds__(kPotThreads) k_potential_fp64(const double *xe, const double *mass, int64_t n,
-                                                                 int64_t jchunk, double eps2, double *phi_part)
+                                                                 double eps2, double *phi_part)
 {
     __shared__ double sx[kPotThreads], sy[kPotThreads], sz[kPotThreads];
     __shared__ p64::Limbs sm[kPotThreads];
     __shared__ int se[kPotThreads];
-    const int64_t i = blockIdx.x * (int64_t)kPotThreads + threadIdx.x;
+    const int64_t T = (n + kPotThreads - 1) / kPotThreads, I = blockIdx.x;
+    const int64_t i = I * kPotThreads + threadIdx.x;
     const int64_t ic = i < n ? i : n - 1;
-    const int64_t j0 = blockIdx.y * jchunk;
-    const int64_t j1 = (j0 + jchunk < n) ? j0 + jchunk : n;
+    // distances 0 .. dmax to the j-tiles
+    const int64_t dmax = (T % 2 == 0 && I >= T / 2) ? T / 2 - 1 : T / 2;
     const double xi = xe[3 * ic], yi = xe[3 * ic + 1], zi = xe[3 * ic + 2];
     const p64::Soft soft2 = p64::soft(eps2);
     p64::Potential acc;
     p64::clear(acc);
-    for (int64_t jb = j0; jb < j1; jb += kPotThreads) {
-        const int64_t j = jb + threadIdx.x;
+    for (int64_t dt = blockIdx.y; dt <= dmax; dt += gridDim.y) {
+        const int64_t J = I + dt < T ? I + dt : I + dt - T;
+        const int64_t j = J * kPotThreads + threadIdx.x;
         __syncthreads();
-        if (j < j1) {
+        if (j < n) {
             sx[threadIdx.x] = xe[3 * j];
             sy[threadIdx.x] = xe[3 * j + 1];
             sz[threadIdx.x] = xe[3 * j + 2];
@@ -382,13 +390,13 @@ __global__ void __launch_bounds__(kPotThreads) k_potential_fp64(const double *xe
             sm[threadIdx.x] = m;
         }
         __syncthreads();
-        const int cnt = (int)((j1 - jb) < kPotThreads ? (j1 - jb) : kPotThreads);
-        const int self = (int)(i - jb >= 0 && i - jb < kPotThreads ? i - jb : -1);
+        const int cnt = (int)(n - J * kPotThreads < kPotThreads ? n - J * kPotThreads : kPotThreads);
+        const int first = dt == 0 ? (int)threadIdx.x + 1 : 0;   // own tile: j > i
         for (int u0 = 0; u0 < cnt; u0 += p64::kFold64) {
             const int u1 = u0 + p64::kFold64 < cnt ? u0 + p64::kFold64 : cnt;
 #pragma unroll 2
             for (int u = u0; u < u1; ++u)
-                p64::pair_potential(sx[u] - xi, sy[u] - yi, sz[u] - zi, sm[u], se[u], u == self, soft2, acc);
+                p64::pair_potential(sx[u] - xi, sy[u] - yi, sz[u] - zi, sm[u], se[u], u < first, soft2, acc);
             p64::fold_fp64(acc);
         }
     }
@@ -446,7 +454,8 @@ __global__ void k_energy_sum(const double *mass, const double *ve, const double 
     }
 }
 
-__global__ void k_energy_final(const double *part2, int g, double *out)
+// side: what a pair counts in sum_i m_i phi_i (-1/2 when both its particles hold it, else -1).
+__global__ void k_energy_final(const double *part2, int g, double side, double *out)
 {
     if (threadIdx.x == 0 && blockIdx.x == 0) {
         double k = 0.0, w = 0.0;
@@ -455,7 +464,7 @@ __global__ void k_energy_final(const double *part2, int g, double *out)
             w += part2[2 * c + 1];
         }
         out[0] = k;
-        out[1] = -0.5 * w;
+        out[1] = side * w;
     }
 }
 
@@ -871,7 +880,7 @@ cudaError_t launch_correct(const State &st, const int32_t *idx, const int64_t *m
 int energy_splits(int64_t n, int num_sms)
 {
     const int64_t itiles = (n + kPotThreads - 1) / kPotThreads;
-    int64_t b = (4 * (int64_t)num_sms + itiles - 1) / itiles;
+    int64_t b = (16 * (int64_t)num_sms + itiles - 1) / itiles;   // CTAs for every SM to even out
     const int64_t jt = (n + kPotThreads - 1) / kPotThreads;
     if (b > jt) b = jt;
     if (b > 64) b = 64;
@@ -883,6 +892,7 @@ cudaError_t launch_energy(bool mixed, const State &st, int64_t n, double t, doub
                           cudaStream_t s)
 {
     k_predict_xv<<<grid_for(n, 256, 1 << 20), 256, 0, s>>>(st, n, t, xe, ve);
+    double side = -0.5;
     int64_t jchunk = (n + nsplit - 1) / nsplit;
     jchunk = (jchunk + kPotThreads - 1) / kPotThreads * kPotThreads;
     dim3 grid((unsigned)((n + kPotThreads - 1) / kPotThreads), (unsigned)nsplit);
@@ -893,10 +903,11 @@ cudaError_t launch_energy(bool mixed, const State &st, int64_t n, double t, doub
     } else if (mixed) {
         k_potential_mixed<<<grid, kPotThreads, 0, s>>>(xe, st.mass, n, jchunk, eps2, phi_part);
     } else {
-        k_potential_fp64<<<grid, kPotThreads, 0, s>>>(xe, st.mass, n, jchunk, eps2, phi_part);
+        k_potential_fp64<<<grid, kPotThreads, 0, s>>>(xe, st.mass, n, eps2, phi_part);
+        side = -1.0;
     }
     k_energy_sum<<<g2, 256, 0, s>>>(st.mass, ve, phi_part, n, nsplit, part2);
-    k_energy_final<<<1, 32, 0, s>>>(part2, g2, out2);
+    k_energy_final<<<1, 32, 0, s>>>(part2, g2, side, out2);
     return cudaGetLastError();
 }
 
