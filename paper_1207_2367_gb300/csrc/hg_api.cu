@@ -40,6 +40,8 @@ struct hg_ctx {
     double *h_stage = nullptr;                     // pinned staging for small uploads
     int32_t *h_flags = nullptr;                    // pinned: (done, err) after two recent replays
     cudaEvent_t ev_flags[2] = {nullptr, nullptr};  // completion of those copies
+    Plan *plan_tab = nullptr;       // graph steps of one system: plans of blocks of 1 .. n <= kPlanTable, or one plan
+    bool plan_tab_valid = false;    // made from the current planner inputs
     double *partial = nullptr;
     int64_t pcap = 0;
     PlanParams pp{};      // evaluation planner inputs
@@ -116,6 +118,11 @@ struct FaultFromEnv {
         }
     }
 } g_fault_from_env;
+
+// Largest system whose graph steps read their plans from a table of all block sizes
+// (48 B each); beyond, where a step's prediction alone takes 35 us and more, a kernel
+// (2 us) scores the candidates of each step's block.
+constexpr int64_t kPlanTable = (int64_t)1 << 20;
 
 constexpr cudaError_t kInjected = cudaErrorUnknown;
 
@@ -201,7 +208,10 @@ EvalArgs eval_args(hg_ctx *c, const int64_t *m_dev, int64_t m_host)
     a.idx = c->d_idx;
     a.m_dev = m_dev;
     a.m_host = m_host;
-    a.plan_dev = m_dev ? reinterpret_cast<const Plan *>(c->d_sc->plan) : nullptr;
+    if (m_dev && c->bv.nc == 0) {   // graph steps of one system
+        a.plan_dev = c->plan_tab;
+        a.plan_stride = c->n <= kPlanTable ? 1 : 0;
+    }
     a.plan_host = m_dev ? Plan{} : make_plan(m_host, c->pp);
     a.partial = c->partial;
     a.eps2 = c->eps * c->eps;
@@ -273,9 +283,10 @@ int upload_scalar(hg_ctx *c, double *dev_field, double v)
 }
 
 // Kernels per graph-replayed block step: one system, selection + prediction,
-// evaluation, reduction, correction (with the next minimum); clusters, three
-// next-block passes, batch plan, prediction, evaluation, reduction, correction.
-int step_kernels(const hg_ctx *c) { return c->bv.nc > 0 ? 8 : 4; }
+// evaluation, reduction + correction (with the next minimum); clusters, two
+// selection passes, batch plan, prediction, evaluation, reduction + correction.
+// Beyond kPlanTable particles the plan is formed in a kernel of its own.
+int step_kernels(const hg_ctx *c) { return c->bv.nc > 0 ? 6 : (c->n > kPlanTable ? 4 : 3); }
 
 // An event record that becomes a graph node when the stream is being captured
 // (a plain record inside a capture only orders work and cannot be timed).
@@ -286,31 +297,32 @@ cudaError_t record_external(cudaEvent_t e, cudaStream_t s)
 
 // One block step (Table 1 sections 1-4 and 8), sizes read on the device.
 // ev: 6 events bracketing the 5 sections, or nullptr.
-// One system: the selection is fused into the prediction (the "next" section
-// is then empty) and the correction leaves the next block time, so a step is
-// four kernels and starts from d_sc->tnext_bits.
-int enqueue_block_step(hg_ctx *c, cudaStream_t s, const cudaEvent_t *ev)
+// One system: the selection is fused into the prediction and the reduction into
+// the correction (the "next" and "reduce" sections are then empty), which leaves
+// the next block time, so a step is three kernels and starts from d_sc->tnext_bits.
+// Clusters: the selection (two passes) and the batch plan come first, six kernels.
+// par: which entries of tnext_bits and slot the step starts from.
+int enqueue_block_step(hg_ctx *c, cudaStream_t s, int par, const cudaEvent_t *ev)
 {
     const bool batch = c->bv.nc > 0;
     if (ev) HG_CUDA(c, record_external(ev[0], s));
     if (batch) {
-        HG_CUDA(c, launch_next_block(c->st, c->n, c->nb_part, c->nb_cnt, c->nb_off, c->d_idx, c->d_sc, 2, c->pp, s));
+        HG_CUDA(c, launch_select_clusters(c->st, c->n, c->nb_cnt, c->nb_off, c->d_idx, c->d_sc, par, c->bv, s));
         HG_CUDA(c, batch_plan(c, &c->d_sc->m, 0, s));
     }
     if (ev) HG_CUDA(c, record_external(ev[1], s));
     if (batch)
         HG_CUDA(c, launch_predict_clusters(c->mixed, c->st, c->rec, c->n, c->bv, &c->d_sc->t_cur, &c->d_sc->m, s));
     else
-        HG_CUDA(c, launch_predict_select(c->mixed, c->st, c->rec, c->n, c->npad, c->d_idx, c->d_sc, 1, c->pp,
-                                         4 * c->num_sms, s));
+        HG_CUDA(c, launch_predict_select(c->mixed, c->st, c->rec, c->n, c->npad, c->d_idx, c->d_sc, par, s));
     if (ev) HG_CUDA(c, record_external(ev[2], s));
-    EvalArgs a = eval_args(c, &c->d_sc->m, 0);
+    const int64_t *m_dev = batch ? &c->d_sc->m : reinterpret_cast<const int64_t *>(&c->d_sc->slot[par]);
+    EvalArgs a = eval_args(c, m_dev, 0);
+    if (!batch && c->n > kPlanTable) HG_CUDA(c, launch_plan_one(c->plan_tab, m_dev, c->pp, s));
     HG_CUDA(c, launch_eval(c->mixed, a, c->num_sms, s));
     if (ev) HG_CUDA(c, record_external(ev[3], s));
-    HG_CUDA(c, launch_reduce(a, c->ra, c->rj, c->rs, 2 * c->num_sms, s));
     if (ev) HG_CUDA(c, record_external(ev[4], s));
-    HG_CUDA(c, launch_correct(c->st, c->d_idx, &c->d_sc->m, 0, c->n, c->ra, c->rj, c->rs, a.rn, step_params(c),
-                              c->d_sc, batch ? 0 : 1, 2 * c->num_sms, s));
+    HG_CUDA(c, launch_reduce_correct(c->st, c->d_idx, c->n, a, step_params(c), c->d_sc, par, 4 * c->num_sms, s));
     if (ev) HG_CUDA(c, record_external(ev[5], s));
     return HG_OK;
 }
@@ -327,11 +339,11 @@ int sync_bound(hg_ctx *c)
     return HG_OK;
 }
 
-// Graph steps of one system start from d_sc->tnext_bits: compute it when the
-// state changed by other means (start-up, hg_set_state, hg_correct).
+// Graph steps start from d_sc->tnext_bits: compute it when the state changed by
+// other means (start-up, hg_set_state, hg_correct).
 int ensure_tnext(hg_ctx *c)
 {
-    if (c->bv.nc > 0 || c->tnext_valid) return HG_OK;
+    if (c->tnext_valid) return HG_OK;
     HG_CUDA(c, launch_next_min(c->st, c->n, c->nb_part, c->d_sc, c->stream));
     c->kernels += 1;
     c->tnext_valid = true;
@@ -348,7 +360,10 @@ int capture(hg_ctx *c, int steps, cudaGraphExec_t *out, std::vector<cudaEvent_t>
     HG_CUDA(c, cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal));
     int rc = HG_OK;
     for (int k = 0; k < steps && rc == HG_OK; ++k)
-        rc = enqueue_block_step(c, c->cap_stream, c->opts.profile ? &ev[(size_t)k * 6] : nullptr);
+        rc = enqueue_block_step(c, c->cap_stream, k & 1, c->opts.profile ? &ev[(size_t)k * 6] : nullptr);
+    // Every graph starts from entry 0: an odd number of steps has left the state in entry 1.
+    if (rc == HG_OK && (steps & 1) && launch_swap_entries(c->d_sc, c->cap_stream) != cudaSuccess)
+        rc = fail(c, HG_ECUDA, "graph capture: launch failed");
     cudaError_t e = cudaStreamEndCapture(c->cap_stream, &g);
     if (rc != HG_OK) {
         if (g) cudaGraphDestroy(g);
@@ -364,6 +379,11 @@ int capture(hg_ctx *c, int steps, cudaGraphExec_t *out, std::vector<cudaEvent_t>
 int ensure_graphs(hg_ctx *c)
 {
     int rc = HG_OK;
+    if (c->bv.nc == 0 && c->n <= kPlanTable && !c->plan_tab_valid) {
+        HG_CUDA(c, launch_plan_table(c->plan_tab, c->n, c->pp, c->stream));
+        c->kernels += 1;
+        c->plan_tab_valid = true;
+    }
     if (!c->g_one) rc = capture(c, 1, &c->g_one, c->ev_one);
     if (rc == HG_OK && !c->g_many) rc = capture(c, c->opts.graph_steps, &c->g_many, c->ev_many);
     return rc;
@@ -374,7 +394,7 @@ int replay(hg_ctx *c, bool many)
 {
     HG_CUDA(c, cudaGraphLaunch(many ? c->g_many : c->g_one, c->stream));
     const int steps = many ? c->opts.graph_steps : 1;
-    c->kernels += (int64_t)step_kernels(c) * steps;
+    c->kernels += (int64_t)step_kernels(c) * steps + (steps & 1);
     if (!c->opts.profile) return HG_OK;
     HG_CUDA(c, cudaStreamSynchronize(c->stream));
     const std::vector<cudaEvent_t> &ev = many ? c->ev_many : c->ev_one;
@@ -511,22 +531,24 @@ int init_impl(hg_ctx *c, const double *mass, const double *pos, const double *ve
         bv.a_off = dalloc<int64_t>(c, nc + 1);
         bv.item_off = dalloc<int64_t>(c, nc + 1);
         bv.part_off = dalloc<int64_t>(c, nc + 1);
-        bv.pred_off = dalloc<int64_t>(c, nc + 1);
+        bv.act = dalloc<int32_t>(c, nc);
         bv.tpi_c = dalloc<int32_t>(c, nc);
         bv.b_c = dalloc<int32_t>(c, nc);
         bv.tps = dalloc<int64_t>(c, 1);
-        if (!clo || !ro || !rm || !co || !bv.a_off || !bv.item_off || !bv.part_off || !bv.pred_off || !bv.tpi_c ||
+        if (!clo || !ro || !rm || !co || !bv.a_off || !bv.item_off || !bv.part_off || !bv.act || !bv.tpi_c ||
             !bv.b_c || !bv.tps)
             return fail(c, HG_ENOMEM, "device allocation failed");
         HG_CUDA(c, cudaMemcpy(clo, c->cl_off_host.data(), (nc + 1) * sizeof(int64_t), cudaMemcpyHostToDevice));
         HG_CUDA(c, cudaMemcpy(ro, rec_off.data(), (nc + 1) * sizeof(int64_t), cudaMemcpyHostToDevice));
         HG_CUDA(c, cudaMemcpy(rm, rmap.data(), n * sizeof(int32_t), cudaMemcpyHostToDevice));
         HG_CUDA(c, cudaMemcpy(co, cl_of.data(), n * sizeof(int32_t), cudaMemcpyHostToDevice));
+        HG_CUDA(c, cudaMemsetAsync(bv.act, 0, (size_t)nc * sizeof(int32_t), c->stream));
         bv.cl_off = clo;
         bv.rec_off = ro;
         bv.rmap = rm;
         bv.cl_of = co;
     }
+    c->plan_tab = dalloc<Plan>(c, nc > 0 || n > kPlanTable ? 1 : n);
     c->partial = dalloc<double>(c, (int64_t)kOut * pcap);
     c->ra = dalloc<double>(c, 3 * n);
     c->rj = dalloc<double>(c, 3 * n);
@@ -541,7 +563,7 @@ int init_impl(hg_ctx *c, const double *mass, const double *pos, const double *ve
     c->e_out = dalloc<double>(c, 2);
     c->l_part = dalloc<double>(c, 3 * c->e_g2);
     c->l_out = dalloc<double>(c, 3);
-    ok = ok && c->d_idx && c->d_idx2 && c->nb_part && c->nb_cnt && c->nb_off && c->d_sc && c->partial && c->ra &&
+    ok = ok && c->d_idx && c->d_idx2 && c->nb_part && c->nb_cnt && c->nb_off && c->d_sc && c->plan_tab && c->partial && c->ra &&
          c->rj && c->rs && c->rn && c->xe && c->ve && c->phi_part && c->e_part && c->e_out && c->l_part && c->l_out;
     if (!ok) return fail(c, HG_ENOMEM, "device allocation failed");
 
@@ -699,6 +721,7 @@ int tune_impl(hg_ctx *c, int64_t m_max, int32_t reps_in, hg_tune_entry *report, 
         return fail(c, HG_ECUDA, "cudaEventCreate failed");
     }
     drop_graphs(c);
+    c->plan_tab_valid = false;
     invalidate(c);
     int rc = HG_OK;
     int32_t count = 0;
@@ -864,8 +887,7 @@ int hg_next_block(hg_ctx *c, double *t_next, int32_t *idx, int64_t cap, int64_t 
     const CallRange range_("hg_next_block");
     if (!c) return HG_EINVAL;
     if (const int rb = sync_bound(c)) return rb;
-    HG_CUDA(c, launch_next_block(c->st, c->n, c->nb_part, c->nb_cnt, c->nb_off, c->d_idx, c->d_sc, 0, c->pp,
-                                 c->stream));
+    HG_CUDA(c, launch_next_block(c->st, c->n, c->nb_part, c->nb_cnt, c->nb_off, c->d_idx, c->d_sc, c->stream));
     c->kernels += 3;
     int rc = sync_scalars(c);
     if (rc) return rc;
@@ -974,8 +996,8 @@ int hg_correct(hg_ctx *c, const int32_t *idx, int64_t m)
         return fail(c, HG_ESTATE, "list differs from the evaluation, or a particle is not due at the block time");
     // 3 lanes per particle, units of 10 particles per warp, 4 warps per CTA
     const int cgrid = (int)std::min<int64_t>(((m + 9) / 10 + 3) / 4, 2 * (int64_t)c->num_sms);
-    HG_CUDA(c, launch_correct(c->st, c->d_idx, nullptr, m, c->n, c->ra, c->rj, c->rs, c->mixed ? c->rn : nullptr,
-                              step_params(c), c->d_sc, 0, cgrid, c->stream));
+    HG_CUDA(c, launch_correct(c->st, c->d_idx, m, c->n, c->ra, c->rj, c->rs, c->mixed ? c->rn : nullptr,
+                              step_params(c), c->d_sc, cgrid, c->stream));
     c->tnext_valid = false;
     c->kernels += 1;
     rc = upload_scalar(c, &c->d_sc->t_cur, c->eval_t);
@@ -1264,6 +1286,7 @@ int hg_tune(hg_ctx *c, int64_t m_max, int32_t reps, hg_tune_entry *report, int32
     int rc = tune_impl(c, m_max, reps, report, cap, n_out);
     if (rc) {
         c->pp = keep;   // a failed run leaves the table as it was
+        c->plan_tab_valid = false;
         drop_graphs(c);
     }
     return rc;
@@ -1326,6 +1349,7 @@ int hg_set_tuning(hg_ctx *c, const int16_t *table)
         if (!ok) return fail(c, HG_EINVAL, "tuning table value out of range for this context");
     }
     for (int k = 0; k < kTuneBuckets; ++k) c->pp.tuned[k] = table[k];
+    c->plan_tab_valid = false;
     drop_graphs(c);
     return HG_OK;
 }

@@ -18,6 +18,7 @@
 
 #include "hg_internal.cuh"
 #include "hg_pair64.cuh"
+#include "hg_plan_dev.cuh"
 
 namespace hg {
 namespace {
@@ -610,6 +611,9 @@ __device__ bool eval_items(const EvalArgs &args, int64_t m, const Plan &pl, unsi
     return true;
 }
 
+// Only this much of a launch is decided here: scoring the planner's candidates in this
+// kernel (even in a function of its own), or one thread unpacking a packed plan into
+// shared memory, cost the pair loops 4 % through the code the compiler made of them.
 template <class P, bool GUARD>
 __global__ void __launch_bounds__(kEvalThreads, P::kMinBlocks) k_eval(const EvalArgs args)
 {
@@ -618,7 +622,7 @@ __global__ void __launch_bounds__(kEvalThreads, P::kMinBlocks) k_eval(const Eval
     double *red = reinterpret_cast<double *>(bars + kStages);
     const int64_t m = args.m_dev ? *args.m_dev : args.m_host;
     if (m <= 0) return;
-    const Plan pl = args.plan_dev ? *args.plan_dev : args.plan_host;
+    const Plan pl = args.plan_dev ? args.plan_dev[(m - 1) * args.plan_stride] : args.plan_host;
     const int64_t n_items = args.bv.nc > 0 ? args.bv.item_off[args.bv.nc] : pl.n_items;
     if ((int64_t)blockIdx.x >= n_items) return;
     if (threadIdx.x == 0) {
@@ -704,9 +708,9 @@ __device__ void reduce_values(const EvalArgs &args, int64_t m, const Plan &pl, d
 
 __global__ void k_reduce(const EvalArgs args, double *ra, double *rj, double *rs)
 {
-    const int64_t m = args.m_dev ? *args.m_dev : args.m_host;
+    const int64_t m = args.m_host;   // explicit calls; graph steps sum in the correction
     if (m <= 0) return;
-    const Plan pl = args.plan_dev ? *args.plan_dev : args.plan_host;
+    const Plan pl = args.plan_host;   // clusters: the work list instead
     reduce_values(args, m, pl, ra, rj, rs, blockIdx.x * (int64_t)blockDim.x + threadIdx.x,
                   (int64_t)gridDim.x * blockDim.x);
 }
@@ -764,12 +768,37 @@ int clip_grid(const EvalArgs &args, int num_sms)
 }
 }  // namespace
 
-int eval_launches(bool, const EvalArgs &) { return 1; }
-
 cudaError_t launch_eval(bool mixed, const EvalArgs &args, int num_sms, cudaStream_t st)
 {
     if (!mixed) return launch_one<F64>(args, clip_grid<F64>(args, num_sms), st);
     return launch_one<MixedEval>(args, clip_grid<MixedEval>(args, num_sms), st);
+}
+
+namespace {
+__global__ void __launch_bounds__(256) k_plan_table(Plan *tab, int64_t n, const __grid_constant__ PlanParams pq)
+{
+    for (int64_t m = blockIdx.x + 1; m <= n; m += gridDim.x) {
+        plan_on_block(m, pq, tab + m - 1);
+        __syncthreads();
+    }
+}
+
+__global__ void __launch_bounds__(256) k_plan_one(Plan *plan, const int64_t *m_dev, const __grid_constant__ PlanParams pq)
+{
+    if (*m_dev > 0) plan_on_block(*m_dev, pq, plan);
+}
+}  // namespace
+
+cudaError_t launch_plan_table(Plan *tab, int64_t n, const PlanParams &pq, cudaStream_t st)
+{
+    k_plan_table<<<(int)(n < 1216 ? n : 1216), 256, 0, st>>>(tab, n, pq);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_plan_one(Plan *plan, const int64_t *m_dev, const PlanParams &pq, cudaStream_t st)
+{
+    k_plan_one<<<1, 256, 0, st>>>(plan, m_dev, pq);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_reduce(const EvalArgs &args, double *ra, double *rj, double *rs, int grid, cudaStream_t st)

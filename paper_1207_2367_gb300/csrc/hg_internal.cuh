@@ -22,11 +22,11 @@ struct DevScalars {
     int32_t done;          // set when a next-block pass found t_next > t_stop
     int32_t err;           // error bits (ERR_*)
     int32_t flag;          // scratch result of validation kernels
-    uint32_t slot;         // active-list entries taken so far by the fused selection
-    int64_t plan[6];       // evaluation plan of the current block (a Plan, written on the device)
-    int64_t tnext_bits;    // bit pattern of min_i tend_i (next-block pass 1, or the last correction)
-    uint32_t arrive[4];    // CTAs done in next-block passes 1 and 2 and in the fused
-                           // selection (the last one resets it); one spare
+    // Graph steps use the two entries of tnext_bits and slot in turn, so that a step's
+    // selection can clear what its correction and the next selection will write.
+    unsigned long long slot[2];   // active-list entries taken by the fused selection
+    int64_t tnext_bits[2];        // bit pattern of min_i tend_i (next-block pass 1, or a correction)
+    uint32_t arrive[4];    // CTAs done in next-block passes 1 and 2 (the last one resets it); two spare
 };
 
 enum : int32_t { ERR_TIMEOUT = 1, ERR_BADIDX = 2, ERR_STATE = 4, ERR_VALUE = 8, ERR_BOUNDS = 16 };
@@ -202,6 +202,20 @@ __host__ __device__ inline int64_t plan_candidate(int64_t m, const PlanParams &q
 
 __host__ __device__ inline int plan_total(const PlanParams &q) { return q.variants * kPlanCandidates; }
 
+// One j-chunk and one thread per i-particle: needs no partial sums, for blocks that no
+// candidate fits (b > 1 chunks of m rows beyond the buffer: a forced j-split, or m near
+// N above 32768 tiles of the longest chunk).
+__host__ __device__ inline Plan plan_unsplit(int64_t m, const PlanParams &q)
+{
+    Plan p{};
+    p.tpi = 1;
+    p.ti = kEvalThreads * q.i_per_thread;
+    p.tiles_per_split = q.ntiles;
+    p.b = 1;
+    p.n_itiles = p.n_items = div_ceil(m > 0 ? m : 1, p.ti);
+    return p;
+}
+
 // The tuned candidate of m's bucket if there is one and it is admissible, else
 // the cheapest admissible candidate of the cost model (ties: lowest index).
 __host__ __device__ inline Plan make_plan(int64_t m, const PlanParams &q)
@@ -217,8 +231,7 @@ __host__ __device__ inline Plan make_plan(int64_t m, const PlanParams &q)
             best = p;
         }
     }
-    if (best_cost < 0) plan_candidate(m, q, 0, best);   // unreachable: candidate 0 is admissible
-    return best;
+    return best_cost >= 0 ? best : plan_unsplit(m, q);
 }
 
 // Independent clusters in one context (nc == 0: a single system).  Particles of
@@ -235,7 +248,7 @@ struct BatchView {
     int64_t *a_off = nullptr;          // [nc+1] first position of each cluster in the active list
     int64_t *item_off = nullptr;       // [nc+1] first work item of each cluster
     int64_t *part_off = nullptr;       // [nc+1] first partial-sum row of each cluster
-    int64_t *pred_off = nullptr;       // [nc+1] prefix of the sizes of clusters with active particles
+    int32_t *act = nullptr;            // [nc] due particles of each cluster (selection to plan, else zero)
     int32_t *tpi_c = nullptr;          // [nc] threads per i-particle
     int32_t *b_c = nullptr;            // [nc] j-chunks
     int64_t *tps = nullptr;            // [1] tiles per j-chunk
@@ -272,10 +285,13 @@ struct EvalArgs {
     int64_t n = 0;                     // particles (bounds of the active list's entries)
     int64_t pcap = 0;                  // rows of the partial-sum buffer
     const int32_t *idx = nullptr;      // active list (device)
-    const int64_t *m_dev = nullptr;    // block size on the device (graph mode), or nullptr
+    const int64_t *m_dev = nullptr;    // block size on the device (clusters, graph steps), or nullptr
     int64_t m_host = 0;                // block size when m_dev == nullptr
-    const Plan *plan_dev = nullptr;    // plan on the device (graph mode), or nullptr
-    Plan plan_host{};                  // plan when plan_dev == nullptr
+    // One system: the plan of a block of m is plan_dev[(m - 1) * plan_stride] (graph
+    // steps: a table of all block sizes, or one plan, stride 0), else plan_host.
+    const Plan *plan_dev = nullptr;
+    int64_t plan_stride = 0;
+    Plan plan_host{};
     double *partial = nullptr;         // [b][m][kOut] partial sums
     double eps2 = 0.0;
     int guard = 0;                     // eps == 0: skip r^2 == 0 pairs
@@ -301,11 +317,11 @@ void set_call_error(const char *msg);
 cudaError_t eval_setup(int device);
 int eval_grid(bool mixed, int num_sms);
 // Evaluation of args: the precision's kernel on min(items, its grid) CTAs with
-// a host plan, on its full persistent grid with a device plan (graph steps) or
-// clusters.
+// a host plan, on its full persistent grid with a device plan or with clusters.
 cudaError_t launch_eval(bool mixed, const EvalArgs &args, int num_sms, cudaStream_t st);
-// Kernels launch_eval issues for a device plan.
-int eval_launches(bool mixed, const EvalArgs &args);
+// Plans of blocks of 1 .. n into tab; the plan of a block of *m_dev > 0 into *plan.
+cudaError_t launch_plan_table(Plan *tab, int64_t n, const PlanParams &pq, cudaStream_t st);
+cudaError_t launch_plan_one(Plan *plan, const int64_t *m_dev, const PlanParams &pq, cudaStream_t st);
 // Sums the b partials of each listed particle into res_{a,j,s} [m][3] and, when
 // args.rn is set, the noise scale into args.rn [m] (grid-stride: grid CTAs of
 // 256 threads, a few per SM).

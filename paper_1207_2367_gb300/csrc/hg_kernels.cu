@@ -13,6 +13,7 @@ namespace hg {
 namespace {
 
 constexpr int kNBThreads = 256;
+constexpr int kSelThreads = 64;   // of the fused selection: small CTAs spread the FP64 work evenly
 
 __device__ __forceinline__ int64_t block_sum_i64(int64_t v, int64_t *sh)
 {
@@ -36,8 +37,9 @@ __device__ __forceinline__ int64_t block_sum_i64(int64_t v, int64_t *sh)
 // IEEE bit pattern orders like its value: the passes compare 64-bit integers.
 // One CTA per contiguous chunk; the last CTA to finish a pass (atomic arrival
 // count, no waiting) completes it: pass 1 the global minimum, pass 2 the
-// chunk offsets, m and the evaluation plan.  Results do not depend on the
-// order in which CTAs run.
+// chunk offsets and m.  Results do not depend on the order in which CTAs run.
+// Graph steps of clusters (graph_step) start at the second pass, with the minimum
+// left by the correction, and also count each cluster's due particles (act).
 // ------------------------------------------------------------------------
 __global__ void __launch_bounds__(kNBThreads) k_nb_min(const double *tend, int64_t n, int64_t chunk,
                                                        long long *part, int g, DevScalars *sc)
@@ -55,21 +57,31 @@ __global__ void __launch_bounds__(kNBThreads) k_nb_min(const double *tend, int64
     v = LLONG_MAX;
     for (int c = threadIdx.x; c < g; c += blockDim.x) v = min(v, *((volatile long long *)part + c));
     v = block_min_ll(v, sh);
-    if (threadIdx.x == 0) sc->tnext_bits = v;
+    if (threadIdx.x == 0) sc->tnext_bits[0] = v;
 }
 
 __global__ void __launch_bounds__(kNBThreads) k_nb_count(const double *tend, int64_t n, int64_t chunk,
                                                          int32_t *cnt, int32_t *off, int g, DevScalars *sc,
-                                                         int count_step, const PlanParams pq)
+                                                         int graph_step, int par, const int32_t *cl_of,
+                                                         int32_t *act)
 {
     __shared__ long long shl[32];
     __shared__ int64_t shi[32];
     __shared__ int last;
-    const long long tn = *((volatile long long *)&sc->tnext_bits);
+    const long long tn = *((volatile long long *)&sc->tnext_bits[par]);
     const long long *bits = reinterpret_cast<const long long *>(tend);
     const int64_t lo = blockIdx.x * chunk, hi = (lo + chunk < n) ? lo + chunk : n;
     int64_t c = 0;
-    for (int64_t i = lo + threadIdx.x; i < hi; i += blockDim.x) c += (__ldg(bits + i) == tn) ? 1 : 0;
+    const bool due_step = __longlong_as_double(tn) <= sc->t_stop;
+    for (int64_t i = lo + threadIdx.x; i < hi; i += blockDim.x)
+        if (__ldcg(bits + i) == tn) {
+            c += 1;
+            if (act && due_step) {   // one atomic per cluster among the lanes here
+                const int cl = cl_of[i];
+                const unsigned same = __match_any_sync(__activemask(), cl);
+                if ((threadIdx.x & 31) == __ffs(same) - 1) atomicAdd(act + cl, __popc(same));
+            }
+        }
     c = block_sum_i64(c, shi);
     if (threadIdx.x == 0) cnt[blockIdx.x] = (int32_t)c;
     if (!last_to_arrive(&sc->arrive[1], (uint32_t)g, &last)) return;
@@ -107,22 +119,20 @@ __global__ void __launch_bounds__(kNBThreads) k_nb_count(const double *tend, int
     }
     const int64_t tot = shl[0];
     const double t_next = __longlong_as_double(tn);
-    const bool take = t_next <= sc->t_stop;
+    const bool take = t_next <= sc->t_stop;   // = due_step
     if (threadIdx.x == 0) {
         if (take) {
             sc->m = tot;
             sc->t_cur = t_next;
             sc->done = 0;
-            if (count_step) {   // 1: count the step and m n interactions; 2: the step only
-                sc->steps += 1;
-                if (count_step == 1) sc->interactions += tot * n;
-            }
+            if (graph_step) sc->steps += 1;
         } else {
             sc->m = 0;
             sc->done = 1;
         }
+        // what the correction gathers into; without a step, what it would have left
+        if (graph_step) sc->tnext_bits[par ^ 1] = take ? LLONG_MAX : tn;
     }
-    if (take) plan_on_block(tot, pq, reinterpret_cast<Plan *>(sc->plan));   // uniform: every thread of the CTA
 }
 
 __global__ void __launch_bounds__(kNBThreads) k_nb_scatter(const double *tend, int64_t n, int64_t chunk,
@@ -130,7 +140,7 @@ __global__ void __launch_bounds__(kNBThreads) k_nb_scatter(const double *tend, i
 {
     __shared__ int32_t woff[33];
     if (*((volatile int64_t *)&sc->m) <= 0) return;
-    const long long tn = *((volatile long long *)&sc->tnext_bits);
+    const long long tn = __double_as_longlong(*((volatile double *)&sc->t_cur));
     const long long *bits = reinterpret_cast<const long long *>(tend);
     int64_t pre = off[blockIdx.x];
     const int64_t lo = blockIdx.x * chunk, hi = (lo + chunk < n) ? lo + chunk : n;
@@ -175,70 +185,58 @@ __global__ void k_predict(const State st, const Records rec, int64_t n, int64_t 
 }
 
 // Clusters, in a block step: only the clusters with active particles need
-// predicted data.  Work index w in [0, pred_off[nc]) is particle
-// cl_off[c] + (w - pred_off[c]) of the cluster c whose range holds w.
+// predicted data.
 template <bool MIXED>
 __global__ void k_predict_clusters(const State st, const Records rec, int64_t n, BatchView bv, const double *t_dev,
                                    const int64_t *m_dev)
 {
     if (*m_dev <= 0) return;
     const double tt = *t_dev;
-    const int64_t total = bv.pred_off[bv.nc];
-    for (int64_t w = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; w < total; w += (int64_t)gridDim.x * blockDim.x) {
-        int lo = 0, hi = bv.nc - 1;   // last cluster with pred_off[c] <= w
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (bv.pred_off[mid] <= w) lo = mid; else hi = mid - 1;
-        }
-        const int64_t i = bv.cl_off[lo] + (w - bv.pred_off[lo]);
-        predict_record<MIXED>(st, rec, i, n, bv.rmap[i], tt);
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        const int c = bv.cl_of[i];
+        if (bv.a_off[c + 1] > bv.a_off[c]) predict_record<MIXED>(st, rec, i, n, bv.rmap[i], tt);
     }
 }
 
 // One system, graph-replayed block steps: Table 1 sections 1 and 2 in one
-// pass.  sc->tnext_bits holds min_i tend_i of the current state (left by the
+// pass.  sc->tnext_bits[par] holds min_i tend_i of the current state (left by the
 // previous correction).  Every thread predicts its records to t_next and the
 // due particles (tend_i == t_next, exact integer compare) are appended to idx
 // with one atomic per warp: the list order is arbitrary, which changes nothing
-// computed (a particle's sums do not depend on its position in the list).  The
-// last CTA to finish (arrival count, no waiting) publishes m, the block time,
-// the counters and the evaluation plan, and clears the minimum for the next
-// correction.  t_next > t_stop: no step (m = 0, done).
+// computed (a particle's sums do not depend on its position in the list); sc->slot[par]
+// counts them.  CTA 0 publishes the block time and clears the other entries for the
+// correction and the next step.  t_next > t_stop: no step (no entries).  (An election
+// of the last CTA to publish the block and score the evaluation's candidate plans, an
+// arrival count on one address and one CTA's work, took half of this pass: 11.4 us at
+// N = 65536 mixed, 5.6 us without.)
 template <bool MIXED>
-__global__ void __launch_bounds__(256) k_predict_select(const State st, const Records rec, int64_t n, int64_t npad,
-                                                       int32_t *idx, DevScalars *sc, int count_step,
-                                                       const PlanParams pq)
+__global__ void __launch_bounds__(kSelThreads) k_predict_select(const State st, const Records rec, int64_t n,
+                                                                int64_t npad, int32_t *idx, DevScalars *sc, int par)
 {
-    __shared__ int last;
-    const long long tn = *((volatile long long *)&sc->tnext_bits);
+    const long long tn = *((volatile long long *)&sc->tnext_bits[par]);
     const double t_next = __longlong_as_double(tn);
-    if (!(t_next <= *((volatile double *)&sc->t_stop))) {
-        if (blockIdx.x == 0 && threadIdx.x == 0) {
+    const bool take = t_next <= *((volatile double *)&sc->t_stop);
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        sc->slot[par ^ 1] = 0ull;
+        sc->tnext_bits[par ^ 1] = take ? LLONG_MAX : tn;
+        sc->done = take ? 0 : 1;
+        if (take) {
+            sc->t_cur = t_next;
+            sc->steps += 1;
+        } else {
             sc->m = 0;
-            sc->done = 1;
         }
-        return;
     }
-    predict_select_pass<MIXED>(st, rec, n, npad, idx, sc, tn, blockIdx.x * (int64_t)blockDim.x + threadIdx.x,
+    if (!take) return;
+    predict_select_pass<MIXED>(st, rec, n, npad, idx, sc, &sc->slot[par], tn, blockIdx.x * (int64_t)blockDim.x + threadIdx.x,
                                (int64_t)gridDim.x * blockDim.x);
-    if (!last_to_arrive(&sc->arrive[2], gridDim.x, &last)) return;
-    __threadfence();
-    // One read of the slot count, shared before thread 0 resets it (a thread
-    // reading it after the reset would score the plan for another m).
-    __shared__ int64_t s_m;
-    if (threadIdx.x == 0) s_m = (int64_t)*((volatile uint32_t *)&sc->slot);
-    __syncthreads();
-    const int64_t m = s_m;
-    if (threadIdx.x == 0) {
-        sc->m = m;
-        sc->t_cur = t_next;
-        sc->done = 0;
-        sc->steps += 1;
-        if (count_step == 1) sc->interactions += m * n;
-        sc->slot = 0u;
-        sc->tnext_bits = LLONG_MAX;
-    }
-    plan_on_block(m > 0 ? m : 1, pq, reinterpret_cast<Plan *>(sc->plan));
+}
+
+// After an odd number of graph steps: entry 0 of the selection's scalars again.
+__global__ void k_swap_entries(DevScalars *sc)
+{
+    sc->tnext_bits[0] = sc->tnext_bits[1];
+    sc->slot[0] = 0ull;
 }
 
 // Predicted FP64 positions and velocities (energy diagnostics).
@@ -278,21 +276,98 @@ __global__ void k_start(State st, int64_t n, const double *ra, const double *rj,
     }
 }
 
-__global__ void __launch_bounds__(128) k_correct(State st, const int32_t *idx, const int64_t *m_dev, int64_t m_host,
+__global__ void __launch_bounds__(128) k_correct(State st, const int32_t *idx, int64_t m,
                                                  const double *ra, const double *rj, const double *rs,
-                                                 const double *rn, StepParams sp, DevScalars *sc, int64_t n,
-                                                 int min_pass)
+                                                 const double *rn, StepParams sp, DevScalars *sc, int64_t n)
 {
-    __shared__ long long sh[32];
-    const int64_t m = m_dev ? *m_dev : m_host;
-    if (m <= 0) return;
     const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, G = (int64_t)gridDim.x * blockDim.x;
-    long long low = LLONG_MAX;
-    if (min_pass) low = scan_min_pass(st, n, __double_as_longlong(*((volatile double *)&sc->t_cur)), g, G);
-    correct_pass(st, idx, m, n, ra, rj, rs, rn, sp, &sc->err, g >> 5, G >> 5, low);
-    if (min_pass) publish_min(sc, low, sh);
+    long long low = LLONG_MAX;   // the host recomputes the minimum before graph steps
+    const ResultArrays res{{ra, rj, rs}, rn};
+    if (sp.order == 4)
+        correct_pass<4>(st, idx, 0, m, n, res, sp, &sc->err, g >> 5, G >> 5, low);
+    else
+        correct_pass<6>(st, idx, 0, m, n, res, sp, &sc->err, g >> 5, G >> 5, low);
 }
 
+// Graph steps: the j-split reduction (Table 1 section 4), the correction of the block
+// and the next block time in one kernel.  A CTA takes chunks of the block:
+// its warps sum the j-chunks' partial rows of the chunk's particles into shared memory
+// (the sums of the reduction kernel, in its order), then correct them.  Small blocks
+// get one particle per CTA, so that the sums of a particle (10 (b / 32 + 5) dependent
+// FP64 instructions of 64 cycles for b j-chunks) use the four FP64 units of an SM of
+// their own.  As two kernels these took 3.9 + 7.3 us of a small block step at N = 65536
+// and a launch more; 10.6 us now (N = 1024 FP64: 3.1 + 6.8, now 7.9).  One copy for each
+// order and for clusters: a launch starts with a cold instruction cache, and the kernel
+// for all of them took 1.3 us more.
+constexpr int kStepThreads = 128;
+constexpr int kStepChunk = kStepThreads / 32 * kCorrUnit;   // particles per chunk, at most
+
+template <int ORDER, bool BATCH>
+__global__ void __launch_bounds__(kStepThreads) k_reduce_correct(State st, const int32_t *idx, int64_t n,
+                                                                 const double *partial, int64_t pcap,
+                                                                 const ResultArrays direct, const BatchView bv,
+                                                                 const Plan *plan, int64_t plan_stride,
+                                                                 StepParams sp, DevScalars *sc, int par)
+{
+    __shared__ long long sh[32];
+    __shared__ double rows[kStepChunk * kOut];
+    const int64_t m = BATCH ? *((volatile int64_t *)&sc->m) : (int64_t)*((volatile unsigned long long *)&sc->slot[par]);
+    if (m <= 0) return;
+    const int b = BATCH ? 0 : plan[(m - 1) * plan_stride].b;   // clusters have their own
+    const int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, G = (int64_t)gridDim.x * blockDim.x;
+    long long low = scan_min_pass(st, n, __double_as_longlong(*((volatile double *)&sc->t_cur)), g, G);
+    if (g == 0 && !BATCH) {
+        sc->m = m;
+        sc->interactions += m * n;
+    }
+    if (b == 1) {                // no j-split: the evaluation wrote the results
+        correct_pass<ORDER>(st, idx, 0, m, n, direct, sp, &sc->err, g >> 5, G >> 5, low);
+    } else if (in_bounds((int64_t)b * m <= pcap, &sc->err)) {
+        const int64_t share = (m + gridDim.x - 1) / gridDim.x;
+        const int64_t P = share < kStepChunk ? share : kStepChunk;
+        const int warp = (int)(threadIdx.x >> 5), lane = (int)(threadIdx.x & 31);
+        for (int64_t q0 = blockIdx.x * P; q0 < m; q0 += gridDim.x * P) {
+            const int cnt = (int)(m - q0 < P ? m - q0 : P);
+            const double *first = partial + q0 * kOut;   // the chunk's values of j-chunk 0: cnt * kOut in a row
+            __syncthreads();
+            if (BATCH) {
+                for (int e = threadIdx.x; e < cnt * kOut; e += kStepThreads) {
+                    const int64_t q = q0 + e / kOut;
+                    const int32_t iq = __ldcg(idx + q);
+                    if (!in_bounds(iq >= 0 && (int64_t)iq < n, &sc->err)) continue;
+                    const int c = bv.cl_of[iq];
+                    const int64_t qb = bv.a_off[c], mc = bv.a_off[c + 1] - qb, row0 = bv.part_off[c] + (q - qb);
+                    const int bc = bv.b_c[c];
+                    if (!in_bounds(row0 >= 0 && row0 + (int64_t)(bc - 1) * mc < pcap, &sc->err)) continue;
+                    const double *first_c = partial + row0 * kOut + e % kOut;
+                    double s = 0.0;
+#pragma unroll 16
+                    for (int sp_ = 0; sp_ < bc; ++sp_) s += __ldcg(first_c + (int64_t)sp_ * mc * kOut);
+                    rows[e] = s;
+                }
+            } else if (b <= 32) {
+                for (int e = threadIdx.x; e < cnt * kOut; e += kStepThreads) {
+                    double s = 0.0;
+#pragma unroll 8
+                    for (int sp_ = 0; sp_ < b; ++sp_) s += __ldcg(first + (int64_t)sp_ * m * kOut + e);
+                    rows[e] = s;
+                }
+            } else {
+                for (int e = warp; e < cnt * kOut; e += kStepThreads / 32) {
+                    double s = 0.0;
+#pragma unroll 4
+                    for (int sp_ = lane; sp_ < b; sp_ += 32) s += __ldcg(first + (int64_t)sp_ * m * kOut + e);
+                    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+                    if (lane == 0) rows[e] = s;
+                }
+            }
+            __syncthreads();
+            correct_pass<ORDER>(st, idx, q0, q0 + cnt, n, ResultRows{rows, q0, direct.rn != nullptr}, sp, &sc->err, warp,
+                         kStepThreads / 32, low);
+        }
+    }
+    publish_min(&sc->tnext_bits[par ^ 1], low, sh);
+}
 
 // ------------------------------------------------------------------------
 // Energy: Sect. 2 softened potential, W = -1/2 sum_i m_i sum_{j != i} m_j /
@@ -619,34 +694,55 @@ __device__ __forceinline__ int batch_tpi(int64_t mc, int ipt, int shift)
     return tpi;
 }
 
+// count (graph steps): the selection has counted each cluster's due particles, and the
+// step's pair evaluations are added to count->interactions; otherwise each cluster's
+// range of the list is found by binary search.  The CTA has a thread per cluster, up to
+// kPlanThreads (64 clusters: 15.4 us with 1024 threads, the search and a scan per
+// candidate, 7.7 us now).
 __global__ void __launch_bounds__(kPlanThreads) k_batch_plan(const int32_t *idx, const int64_t *m_dev, int64_t m_host,
-                                                             BatchView bv, PlanParams q, DevScalars *count)
+                                                             BatchView bv, const __grid_constant__ PlanParams q,
+                                                             DevScalars *count)
 {
     __shared__ int64_t sh[33];
     __shared__ int64_t s_tps;
+    __shared__ unsigned long long s_tot[2 * kTpsCand];
     const int64_t m = m_dev ? *m_dev : m_host;
     if (m <= 0) return;
     const int nc = bv.nc;
-    const int tj = q.tj, ipt = q.i_per_thread, grid = q.grid;
+    const int tj_log = 31 - __clz(q.tj), ipt = q.i_per_thread, grid = q.grid;   // tj a power of two
     const int64_t pcap = q.pcap;
     const BatchKnobs kn = batch_knobs(m, q);
-    for (int c = threadIdx.x; c <= nc; c += blockDim.x) {
-        if (c == nc) {
-            bv.a_off[nc] = m;
-            continue;
-        }
-        const int64_t key = bv.cl_off[c];
-        int64_t lo = 0, hi = m;   // first position with idx >= key
-        while (lo < hi) {
-            const int64_t mid = (lo + hi) >> 1;
-            if (idx[mid] < key) lo = mid + 1; else hi = mid;
-        }
-        bv.a_off[c] = lo;
-    }
-    __syncthreads();
-    // This thread's clusters [c0, c1): active counts and tiles.
+    // This thread's clusters [c0, c1).
     const int per = (nc + (int)blockDim.x - 1) / (int)blockDim.x;
     const int c0 = threadIdx.x * per, c1 = (c0 + per < nc) ? c0 + per : nc;
+    if (threadIdx.x < 2 * kTpsCand) s_tot[threadIdx.x] = 0ull;
+    if (count) {
+        int64_t mine = 0, before, all;
+        for (int c = c0; c < c1; ++c) mine += bv.act[c];
+        block_exscan_i64(mine, sh, before, all);
+        for (int c = c0; c < c1; ++c) {
+            bv.a_off[c] = before;
+            before += bv.act[c];
+            bv.act[c] = 0;
+        }
+        if (threadIdx.x == 0) bv.a_off[nc] = m;
+    } else {
+        for (int c = threadIdx.x; c <= nc; c += blockDim.x) {
+            if (c == nc) {
+                bv.a_off[nc] = m;
+                continue;
+            }
+            const int64_t key = bv.cl_off[c];
+            int64_t lo = 0, hi = m;   // first position with idx >= key
+            while (lo < hi) {
+                const int64_t mid = (lo + hi) >> 1;
+                if (idx[mid] < key) lo = mid + 1; else hi = mid;
+            }
+            bv.a_off[c] = lo;
+        }
+    }
+    __syncthreads();
+    // Active counts and tiles.
     int64_t items[kTpsCand], parts[kTpsCand];
     for (int k = 0; k < kTpsCand; ++k) items[k] = parts[k] = 0;
     for (int c = c0; c < c1; ++c) {
@@ -654,8 +750,8 @@ __global__ void __launch_bounds__(kPlanThreads) k_batch_plan(const int32_t *idx,
         if (mc == 0) continue;
         const int tpi = batch_tpi(mc, ipt, kn.tpi_shift);
         const int64_t ti = kEvalThreads / tpi * ipt;
-        const int64_t nit = (mc + ti - 1) / ti;
-        const int64_t ntc = (bv.rec_off[c + 1] - bv.rec_off[c]) / tj;
+        const int64_t nit = div_ceil(mc, ti);
+        const int64_t ntc = (bv.rec_off[c + 1] - bv.rec_off[c]) >> tj_log;
         for (int k = 0; k < kTpsCand; ++k) {
             const int64_t b = (ntc + (1 << k) - 1) >> k;
             items[k] += nit * b;
@@ -663,18 +759,24 @@ __global__ void __launch_bounds__(kPlanThreads) k_batch_plan(const int32_t *idx,
         }
     }
     for (int k = 0; k < kTpsCand; ++k) {
-        int64_t e, t;
-        block_exscan_i64(items[k], sh, e, t);
-        items[k] = t;
-        block_exscan_i64(parts[k], sh, e, t);
-        parts[k] = t;
+        int64_t a = items[k], b = parts[k];
+        for (int o = 16; o > 0; o >>= 1) {
+            a += __shfl_xor_sync(0xffffffffu, a, o);
+            b += __shfl_xor_sync(0xffffffffu, b, o);
+        }
+        if ((threadIdx.x & 31) == 0) {
+            atomicAdd(&s_tot[k], (unsigned long long)a);
+            atomicAdd(&s_tot[kTpsCand + k], (unsigned long long)b);
+        }
     }
+    __syncthreads();
     if (threadIdx.x == 0) {
+        const int64_t *tot_items = reinterpret_cast<const int64_t *>(s_tot), *tot_parts = tot_items + kTpsCand;
         int pick = -1;
         for (int k = kTpsCand - 1; k >= 0 && pick < 0; --k)
-            if (parts[k] <= pcap && items[k] >= ((int64_t)grid << kn.w_log)) pick = k;
+            if (tot_parts[k] <= pcap && tot_items[k] >= ((int64_t)grid << kn.w_log)) pick = k;
         for (int k = 0; k < kTpsCand && pick < 0; ++k)
-            if (parts[k] <= pcap) pick = k;
+            if (tot_parts[k] <= pcap) pick = k;
         if (pick < 0) pick = kTpsCand - 1;
         s_tps = (int64_t)1 << pick;
         *bv.tps = s_tps;
@@ -686,23 +788,15 @@ __global__ void __launch_bounds__(kPlanThreads) k_batch_plan(const int32_t *idx,
         const int64_t mc = bv.a_off[c + 1] - bv.a_off[c];
         const int tpi = mc > 0 ? batch_tpi(mc, ipt, kn.tpi_shift) : 1;
         const int64_t ti = kEvalThreads / tpi * ipt;
-        const int64_t nit = (mc + ti - 1) / ti;
-        const int64_t ntc = (bv.rec_off[c + 1] - bv.rec_off[c]) / tj;
-        const int64_t b = (ntc + tps - 1) / tps;
+        const int64_t nit = div_ceil(mc, ti);
+        const int64_t ntc = (bv.rec_off[c + 1] - bv.rec_off[c]) >> tj_log;
+        const int64_t b = div_ceil(ntc, tps);
         bv.tpi_c[c] = tpi;
         bv.b_c[c] = (int32_t)b;
         my_items += nit * b;
         my_parts += b * mc;
     }
-    int64_t ie, it, pe, pt, we, wt, my_pred = 0;
-    for (int c = c0; c < c1; ++c)
-        if (bv.a_off[c + 1] > bv.a_off[c]) my_pred += bv.cl_off[c + 1] - bv.cl_off[c];
-    block_exscan_i64(my_pred, sh, we, wt);
-    for (int c = c0; c < c1; ++c) {
-        bv.pred_off[c] = we;
-        if (bv.a_off[c + 1] > bv.a_off[c]) we += bv.cl_off[c + 1] - bv.cl_off[c];
-    }
-    if (threadIdx.x == 0) bv.pred_off[nc] = wt;
+    int64_t ie, it, pe, pt;
     block_exscan_i64(my_items, sh, ie, it);
     block_exscan_i64(my_parts, sh, pe, pt);
     if (count) {   // pair evaluations of this block step: sum over clusters of m_c N_c
@@ -716,7 +810,7 @@ __global__ void __launch_bounds__(kPlanThreads) k_batch_plan(const int32_t *idx,
     for (int c = c0; c < c1; ++c) {
         const int64_t mc = bv.a_off[c + 1] - bv.a_off[c];
         const int64_t ti = kEvalThreads / bv.tpi_c[c] * ipt;
-        const int64_t nit = (mc + ti - 1) / ti;
+        const int64_t nit = div_ceil(mc, ti);
         bv.item_off[c] = ie;
         bv.part_off[c] = pe;
         ie += nit * bv.b_c[c];
@@ -778,12 +872,21 @@ inline int grid_for(int64_t work, int threads, int cap)
 int nb_grid(int64_t n) { return (int)((n + kNBChunk - 1) / kNBChunk); }
 
 cudaError_t launch_next_block(const State &st, int64_t n, double *part, int32_t *cnt, int32_t *off, int32_t *idx,
-                              DevScalars *sc, int count_step, const PlanParams &pq, cudaStream_t s)
+                              DevScalars *sc, cudaStream_t s)
 {
     const int g = nb_grid(n);
     long long *bits = reinterpret_cast<long long *>(part);
     k_nb_min<<<g, kNBThreads, 0, s>>>(st.tend, n, kNBChunk, bits, g, sc);
-    k_nb_count<<<g, kNBThreads, 0, s>>>(st.tend, n, kNBChunk, cnt, off, g, sc, count_step, pq);
+    k_nb_count<<<g, kNBThreads, 0, s>>>(st.tend, n, kNBChunk, cnt, off, g, sc, 0, 0, nullptr, nullptr);
+    k_nb_scatter<<<g, kNBThreads, 0, s>>>(st.tend, n, kNBChunk, off, idx, sc);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_select_clusters(const State &st, int64_t n, int32_t *cnt, int32_t *off, int32_t *idx,
+                                   DevScalars *sc, int par, const BatchView &bv, cudaStream_t s)
+{
+    const int g = nb_grid(n);
+    k_nb_count<<<g, kNBThreads, 0, s>>>(st.tend, n, kNBChunk, cnt, off, g, sc, 1, par, bv.cl_of, bv.act);
     k_nb_scatter<<<g, kNBThreads, 0, s>>>(st.tend, n, kNBChunk, off, idx, sc);
     return cudaGetLastError();
 }
@@ -821,17 +924,19 @@ cudaError_t launch_predict(bool mixed, const State &st, const Records &rec, int6
 }
 
 cudaError_t launch_predict_select(bool mixed, const State &st, const Records &rec, int64_t n, int64_t npad,
-                                  int32_t *idx, DevScalars *sc, int count_step, const PlanParams &pq, int max_grid,
-                                  cudaStream_t s)
+                                  int32_t *idx, DevScalars *sc, int par, cudaStream_t s)
 {
-    // Persistent grid: every CTA takes one atomic on the arrival counter, and
-    // at N = 2^20 sixteen thousand of them on one address cost more than the
-    // prediction itself.
-    const int g = grid_for(npad, 256, max_grid);
+    const int g = grid_for(npad, kSelThreads, 1 << 20);
     if (mixed)
-        k_predict_select<true><<<g, 256, 0, s>>>(st, rec, n, npad, idx, sc, count_step, pq);
+        k_predict_select<true><<<g, kSelThreads, 0, s>>>(st, rec, n, npad, idx, sc, par);
     else
-        k_predict_select<false><<<g, 256, 0, s>>>(st, rec, n, npad, idx, sc, count_step, pq);
+        k_predict_select<false><<<g, kSelThreads, 0, s>>>(st, rec, n, npad, idx, sc, par);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_swap_entries(DevScalars *sc, cudaStream_t s)
+{
+    k_swap_entries<<<1, 1, 0, s>>>(sc);
     return cudaGetLastError();
 }
 
@@ -858,7 +963,8 @@ cudaError_t launch_pad_records(bool mixed, const Records &rec, int64_t npad, cud
 cudaError_t launch_batch_plan(const int32_t *idx, const int64_t *m_dev, int64_t m_host, const BatchView &bv,
                               const PlanParams &q, DevScalars *count, cudaStream_t s)
 {
-    k_batch_plan<<<1, kPlanThreads, 0, s>>>(idx, m_dev, m_host, bv, q, count);
+    const int threads = bv.nc < kPlanThreads ? (bv.nc + 31) / 32 * 32 : kPlanThreads;
+    k_batch_plan<<<1, threads, 0, s>>>(idx, m_dev, m_host, bv, q, count);
     return cudaGetLastError();
 }
 
@@ -869,11 +975,25 @@ cudaError_t launch_start(const State &st, int64_t n, const double *ra, const dou
     return cudaGetLastError();
 }
 
-cudaError_t launch_correct(const State &st, const int32_t *idx, const int64_t *m_dev, int64_t m_host, int64_t n,
+cudaError_t launch_correct(const State &st, const int32_t *idx, int64_t m, int64_t n,
                            const double *ra, const double *rj, const double *rs, const double *rn,
-                           const StepParams &sp, DevScalars *sc, int min_pass, int grid, cudaStream_t s)
+                           const StepParams &sp, DevScalars *sc, int grid, cudaStream_t s)
 {
-    k_correct<<<grid, 128, 0, s>>>(st, idx, m_dev, m_host, ra, rj, rs, rn, sp, sc, n, min_pass);
+    k_correct<<<grid, 128, 0, s>>>(st, idx, m, ra, rj, rs, rn, sp, sc, n);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_reduce_correct(const State &st, const int32_t *idx, int64_t n, const EvalArgs &a,
+                                  const StepParams &sp, DevScalars *sc, int par, int grid, cudaStream_t s)
+{
+    auto launch = [&](auto kernel) {
+        kernel<<<grid, kStepThreads, 0, s>>>(st, idx, n, a.partial, a.pcap, ResultArrays{{a.ra, a.rj, a.rs}, a.rn},
+                                             a.bv, a.plan_dev, a.plan_stride, sp, sc, par);
+    };
+    if (a.bv.nc > 0)
+        sp.order == 4 ? launch(k_reduce_correct<4, true>) : launch(k_reduce_correct<6, true>);
+    else
+        sp.order == 4 ? launch(k_reduce_correct<4, false>) : launch(k_reduce_correct<6, false>);
     return cudaGetLastError();
 }
 

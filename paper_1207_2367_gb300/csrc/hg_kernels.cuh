@@ -21,16 +21,21 @@ constexpr int64_t kNBChunk = 2048;   // particles per CTA in the next-block pass
 int nb_grid(int64_t n);
 // part, cnt, off: nb_grid(n) entries each.
 cudaError_t launch_next_block(const State &st, int64_t n, double *part, int32_t *cnt, int32_t *off, int32_t *idx,
-                              DevScalars *sc, int count_step, const PlanParams &pq, cudaStream_t s);
-// Pass 1 alone: sc->tnext_bits = bits of min_i tend_i.
+                              DevScalars *sc, cudaStream_t s);
+// Graph steps of clusters: the list of the particles due at sc->tnext_bits[par] (kept by
+// launch_reduce_correct), ascending, and the due particles of each cluster in bv.act.
+cudaError_t launch_select_clusters(const State &st, int64_t n, int32_t *cnt, int32_t *off, int32_t *idx,
+                                   DevScalars *sc, int par, const BatchView &bv, cudaStream_t s);
+// Pass 1 alone: sc->tnext_bits[0] = bits of min_i tend_i.
 cudaError_t launch_next_min(const State &st, int64_t n, double *part, DevScalars *sc, cudaStream_t s);
 // One system, graph-replayed block steps: block selection fused into the
-// prediction.  Needs sc->tnext_bits = min_i tend_i (kept by launch_correct with
-// min_pass); predicts every record to t_next, lists the due particles in idx
-// (arbitrary order), sets m, t_cur, done, the counters and the plan.
+// prediction.  Needs sc->tnext_bits[par] = min_i tend_i and sc->slot[par] = 0 (kept
+// by the previous step, par ^ 1); predicts every record to t_next and lists the due
+// particles in idx (arbitrary order), sc->slot[par] of them.
 cudaError_t launch_predict_select(bool mixed, const State &st, const Records &rec, int64_t n, int64_t npad,
-                                  int32_t *idx, DevScalars *sc, int count_step, const PlanParams &pq, int max_grid,
-                                  cudaStream_t s);
+                                  int32_t *idx, DevScalars *sc, int par, cudaStream_t s);
+// After an odd number of graph steps: the next one starts from entry 0 again.
+cudaError_t launch_swap_entries(DevScalars *sc, cudaStream_t s);
 // After the state was replaced: tend = t + dt and the FP32 copies (st.f32).
 cudaError_t launch_tend(const State &st, int64_t n, cudaStream_t s);
 // The FP32 copies alone (a no-op for FP64 contexts, st.f32 == nullptr).
@@ -52,14 +57,17 @@ cudaError_t launch_batch_plan(const int32_t *idx, const int64_t *m_dev, int64_t 
                               const PlanParams &q, DevScalars *count, cudaStream_t s);
 cudaError_t launch_start(const State &st, int64_t n, const double *ra, const double *rj, const double *rs,
                          const StepParams &sp, cudaStream_t s);
-// Corrector and new steps of the listed particles.  min_pass (graph steps of
-// one system, where the list is every particle due at sc->t_cur): also leave
-// min_i tend_i of the new state in sc->tnext_bits (reset beforehand by the
-// selection).  rn: noise scale of each listed particle (mixed), or nullptr
-// (the noise floor then scales with |a1|).  grid: CTAs of 128 threads.
-cudaError_t launch_correct(const State &st, const int32_t *idx, const int64_t *m_dev, int64_t m_host, int64_t n,
+// Corrector and new steps of the listed particles.  rn: noise scale of each listed
+// particle (mixed), or nullptr (the noise floor then scales with |a1|).  grid: CTAs
+// of 128 threads.
+cudaError_t launch_correct(const State &st, const int32_t *idx, int64_t m, int64_t n,
                            const double *ra, const double *rj, const double *rs, const double *rn,
-                           const StepParams &sp, DevScalars *sc, int min_pass, int grid, cudaStream_t s);
+                           const StepParams &sp, DevScalars *sc, int grid, cudaStream_t s);
+// Graph steps (the list is every particle due at sc->t_cur): the sums of
+// the evaluation a's j-chunks, the correction, and min_i tend_i of the new state in
+// sc->tnext_bits[par ^ 1] (reset beforehand by the selection).
+cudaError_t launch_reduce_correct(const State &st, const int32_t *idx, int64_t n, const EvalArgs &a,
+                                  const StepParams &sp, DevScalars *sc, int par, int grid, cudaStream_t s);
 int energy_splits(int64_t n, int num_sms);
 cudaError_t launch_energy(bool mixed, const State &st, int64_t n, double t, double eps2, double *xe, double *ve,
                           double *phi_part, int nsplit, double *part2, int g2, double *out2, const BatchView &bv,

@@ -289,6 +289,13 @@ HG_P64 void add_term(Sums &a, int g, Limbs q, const Limbs (&x)[3])
     }
 }
 
+// (H, M) 2^-d; from d = 32 on the rest below H's last place is dropped.
+HG_P64 void shift_sum(int64_t &H, uint32_t &M, int d)
+{
+    M = d < 32 ? (uint32_t)lo32((int64_t)shr((uint64_t)word(lo32(H), (int32_t)M), d)) : 0u;
+    H = sar(H, d);
+}
+
 // A term larger than the sums' units allow moves them to its exponent.
 HG_P64 void raise(Sums &a, const int (&need)[3])
 {
@@ -298,11 +305,7 @@ HG_P64 void raise(Sums &a, const int (&need)[3])
         a.E[g] += d;
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
-            int64_t &H = a.H[3 * g + k];
-            uint32_t &M = a.M[3 * g + k];
-            // (H, M) 2^-d; from d = 32 on the rest below H's last place is dropped
-            M = d < 32 ? (uint32_t)lo32((int64_t)shr((uint64_t)word(lo32(H), (int32_t)M), d)) : 0u;
-            H = sar(H, d);
+            shift_sum(a.H[3 * g + k], a.M[3 * g + k], d);
         }
     }
 }

@@ -224,7 +224,6 @@ extern "C" int hg_evaluate_static(int64_t n, const double *mass, const double *p
     a.idx = idx;
     a.m_dev = nullptr;
     a.m_host = m;
-    a.plan_dev = nullptr;
     const PlanParams pq = plan_params(mixed, npad, slot->sms, kStaticPcap, 0, 0);
     a.plan_host = make_plan(m, pq);
     a.partial = reinterpret_cast<double *>(base + kRecBytes);

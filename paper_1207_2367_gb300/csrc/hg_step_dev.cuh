@@ -1,6 +1,5 @@
-// hg_step_dev.cuh -- device code of the block step (hg_kernels.cu): the
-// evaluation planner on one CTA, CTA reductions and arrival counts, the FP64
-// predictor (Sect. 3 item 1), the corrector with the Hermite interpolation and
+// hg_step_dev.cuh -- device code of the block step (hg_kernels.cu): CTA
+// reductions and arrival counts, the FP64 predictor (Sect. 3 item 1), the corrector with the Hermite interpolation and
 // the step criterion (Sect. 3 item 3, criterion equations, power-of-two
 // blocks), and the passes of a graph-replayed block step.
 #pragma once
@@ -11,6 +10,7 @@
 #include <stdint.h>
 
 #include "hg_kernels.cuh"
+#include "hg_plan_dev.cuh"
 
 namespace hg {
 namespace {
@@ -30,59 +30,6 @@ __device__ __forceinline__ long long block_min_ll(long long v, long long *sh)
     __syncthreads();
     return sh[0];
 }
-
-// The evaluation plan for block size m, by every thread of one CTA (at least
-// kPlanCandidates threads would score one candidate each; fewer loop): the
-// lowest cost wins, ties to the lowest candidate index (make_plan's choice on
-// the host).  A tuned candidate of m's bucket that is admissible wins outright.
-// Thread 0 writes *out (global or shared memory).
-__device__ void plan_on_block(int64_t m, const PlanParams &q, Plan *out)
-{
-    __shared__ int64_t s_cost[32];
-    __shared__ int s_cand[32];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = (int)(blockDim.x >> 5);
-    Plan p;
-    const int tc = q.tuned[tune_bucket(m)];
-    if (tc >= 0 && plan_candidate(m, q, tc, p) >= 0) {   // measured choice
-        if (threadIdx.x == 0) *out = p;
-        return;
-    }
-    int64_t best = -1;
-    int bc = 0x7fffffff;
-    for (int c = threadIdx.x; c < plan_total(q); c += blockDim.x) {
-        const int64_t cost = plan_candidate(m, q, c, p);
-        if (cost >= 0 && (best < 0 || cost < best)) {
-            best = cost;
-            bc = c;
-        }
-    }
-    for (int off = 16; off > 0; off >>= 1) {
-        const int64_t ob = __shfl_xor_sync(0xffffffffu, best, off);
-        const int oc = __shfl_xor_sync(0xffffffffu, bc, off);
-        if (ob >= 0 && (best < 0 || ob < best || (ob == best && oc < bc))) {
-            best = ob;
-            bc = oc;
-        }
-    }
-    if (lane == 0) {
-        s_cost[w] = best;
-        s_cand[w] = bc;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int k = 1; k < nw; ++k) {
-            const int64_t ob = s_cost[k];
-            const int oc = s_cand[k];
-            if (ob >= 0 && (best < 0 || ob < best || (ob == best && oc < bc))) {
-                best = ob;
-                bc = oc;
-            }
-        }
-        plan_candidate(m, q, best >= 0 ? bc : 0, p);
-        *out = p;
-    }
-}
-
 
 // True in every thread of the CTA that arrives last (counter reset for reuse).
 __device__ __forceinline__ bool last_to_arrive(uint32_t *counter, uint32_t total, int *sh_flag)
@@ -477,24 +424,21 @@ __device__ __forceinline__ bool multiple_of_pow2(double t1, int p)
 
 __device__ __forceinline__ double sq3(const double *p) { return p[0] * p[0] + p[1] * p[1] + p[2] * p[2]; }
 
-// New time t0 + h and p = 6 step of particle i from d = a^(0..5) at the step's end.
-// A: the acceleration change left after a0 + j0 h + s0 h^2/2 (a0 + j0 h for
+// New time t0 + h and p = 6 step of particle i from d = a^(0..5) at the step's end
+// (qn: their squared norms).  qA: squared norm of the acceleration change left after a0 + j0 h + s0 h^2/2 (a0 + j0 h for
 // p = 4).  Below the noise floor of the evaluation, sp.noise_rel times the
 // noise scale (sum_j m_j / r_ij^2 where the evaluation provides it, else |a1|;
 // compared as squares), the interpolated derivatives are noise and the
 // criterion may not shrink the step.
 template <int P>
 __device__ __forceinline__ double finish_step(const State &st, int64_t i, double t0, double h, int e, bool pow2,
-                                              const double (*d)[3], const double *A, double scale2,
+                                              const double (*d)[3], const double *qn, double qA, double scale2,
                                               const StepParams &sp, bool store)
 {
     const double t1 = t0 + h;
-    const bool noisy = sp.noise_rel > 0.0 && sq3(A) < (sp.noise_rel * sp.noise_rel) * scale2;
+    const bool noisy = sp.noise_rel > 0.0 && qA < (sp.noise_rel * sp.noise_rel) * scale2;
     double dt1;
     int F, kmin, kmax;
-    double qn[P];
-#pragma unroll
-    for (int s = 0; s < P; ++s) qn[s] = sq3(d[s]);
     if (pow2 && pow2_exponent(sp.dt_min, kmin) && pow2_exponent(sp.dt_max, kmax) &&
         (noisy || criterion_floor_log2<P>(qn, sp.log2_eta, F))) {
         // The power-of-two rule (block_dt) on exponents: shrink to max(F, k_min)
@@ -529,13 +473,30 @@ __device__ __forceinline__ double finish_step(const State &st, int64_t i, double
 // instructions of a small block is a third of the one-thread-per-particle form.
 constexpr int kCorrUnit = 10;
 
-template <int P>
-__device__ __forceinline__ void correct_lane(const State &st, const int32_t *idx, const double *ra, const double *rj,
-                                             const double *rs, const double *rn, const StepParams &sp, int64_t m, int64_t n, int32_t *err,
-                                             int64_t u, long long &low)
+// Component k of particle q's evaluated derivative d (0: acceleration, 1: jerk, 2: snap)
+// and its noise scale, from the arrays [m][3] (noise [m], or nullptr) ...
+struct ResultArrays {
+    const double *r[3], *rn;
+    __device__ __forceinline__ double at(int d, int64_t q, int k) const { return __ldcg(r[d] + 3 * q + k); }
+    __device__ __forceinline__ double noise(int64_t q) const { return rn ? __ldcg(rn + q) : 0.0; }
+    __device__ __forceinline__ bool has_noise() const { return rn != nullptr; }
+};
+// ... or from rows of kOut values in shared memory, the first being particle q0's.
+struct ResultRows {
+    const double *row;
+    int64_t q0;
+    bool noisy;
+    __device__ __forceinline__ double at(int d, int64_t q, int k) const { return row[(q - q0) * kOut + 3 * d + k]; }
+    __device__ __forceinline__ double noise(int64_t q) const { return row[(q - q0) * kOut + 9]; }
+    __device__ __forceinline__ bool has_noise() const { return noisy; }
+};
+
+template <int P, class R>
+__device__ __forceinline__ void correct_lane(const State &st, const int32_t *idx, const R &res, const StepParams &sp,
+                                             int64_t m, int64_t n, int32_t *err, int64_t q_first, long long &low)
 {
     const int lane = threadIdx.x & 31, sub = lane / 3, k = lane - 3 * sub;
-    const int64_t q = u * kCorrUnit + sub;
+    const int64_t q = q_first + sub;
     bool act = sub < kCorrUnit && q < m;
     // What is indexed by the list position q is loaded at once, then the
     // particle's own fields in one more round trip: the chain of dependent
@@ -544,10 +505,10 @@ __device__ __forceinline__ void correct_lane(const State &st, const int32_t *idx
     double dk[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0}, rnq = 0.0;
     if (act) {
         iq = __ldcg(idx + q);
-        dk[0] = __ldcg(ra + 3 * q + k);
-        dk[1] = __ldcg(rj + 3 * q + k);
-        if (P == 6) dk[2] = __ldcg(rs + 3 * q + k);
-        if (rn) rnq = __ldcg(rn + q);
+        dk[0] = res.at(0, q, k);
+        dk[1] = res.at(1, q, k);
+        if (P == 6) dk[2] = res.at(2, q, k);
+        if (res.has_noise()) rnq = res.noise(q);
     }
     if (act && !in_bounds(iq >= 0 && (int64_t)iq < n, err)) act = false;
     double Ak = 0.0, h = 1.0, t0 = 0.0;
@@ -580,9 +541,31 @@ __device__ __forceinline__ void correct_lane(const State &st, const int32_t *idx
         for (int r = 0; r < P; ++r) d[r][c] = __shfl_sync(0xffffffffu, dk[r], src);
         A[c] = __shfl_sync(0xffffffffu, Ak, src);
     }
+    // The squared norms of the P vectors and of A: each lane of the triple forms those of
+    // vectors k, k + 3, ... (three of 64-cycle FP64 instructions each, one lane's values
+    // or three's at the same cost), then all get all.
+    constexpr int kOwn = P / 3 + 1;   // P = 6: 0..5 and A; P = 4: 0..3, A, one spare
+    double own[kOwn], qn[3 * kOwn];
+#pragma unroll
+    for (int r = 0; r < kOwn; ++r) {
+        double v[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            const double v0 = 3 * r < P ? d[3 * r < P ? 3 * r : 0][c] : A[c];
+            const double v1 = 3 * r + 1 < P ? d[3 * r + 1 < P ? 3 * r + 1 : 0][c] : A[c];
+            const double v2 = 3 * r + 2 < P ? d[3 * r + 2 < P ? 3 * r + 2 : 0][c] : A[c];
+            v[c] = k == 0 ? v0 : (k == 1 ? v1 : v2);
+        }
+        own[r] = sq3(v);
+    }
+#pragma unroll
+    for (int s = 0; s < 3 * kOwn; ++s) {
+        const int src = base + s % 3 < 32 ? base + s % 3 : 31;
+        qn[s] = __shfl_sync(0xffffffffu, own[s / 3], src);
+    }
     if (act) {
-        const double scale2 = rn ? rnq * rnq : sq3(d[0]);
-        low = min(low, __double_as_longlong(finish_step<P>(st, i, t0, h, e, pow2, d, A, scale2, sp, k == 0)));
+        const double scale2 = res.has_noise() ? rnq * rnq : qn[0];
+        low = min(low, __double_as_longlong(finish_step<P>(st, i, t0, h, e, pow2, d, qn, qn[P], scale2, sp, k == 0)));
     }
 }
 
@@ -596,11 +579,11 @@ __device__ __forceinline__ void correct_lane(const State &st, const int32_t *idx
 
 // Table 1 sections 1-2 in one pass: predict every record to t_next (bit
 // pattern tn) and append each particle with tend_i == t_next to idx, one
-// atomic on sc->slot per warp (the list order is arbitrary: a particle's sums
+// atomic on *slot per warp (the list order is arbitrary: a particle's sums
 // do not depend on its position).  Whole warps take part (the ballot).
 template <bool MIXED>
 __device__ void predict_select_pass(const State &st, const Records &rec, int64_t n, int64_t npad, int32_t *idx,
-                                    DevScalars *sc, long long tn, int64_t g0, int64_t G)
+                                    DevScalars *sc, unsigned long long *slot, long long tn, int64_t g0, int64_t G)
 {
     const double t_next = __longlong_as_double(tn);
     const long long *bits = reinterpret_cast<const long long *>(st.tend);
@@ -611,8 +594,8 @@ __device__ void predict_select_pass(const State &st, const Records &rec, int64_t
         const bool due = i < n && __ldcg(bits + i) == tn;
         const unsigned ball = __ballot_sync(0xffffffffu, due);
         if (ball) {
-            uint32_t b0 = 0;
-            if (l == 0) b0 = atomicAdd(&sc->slot, (uint32_t)__popc(ball));
+            unsigned long long b0 = 0;
+            if (l == 0) b0 = atomicAdd(slot, (unsigned long long)__popc(ball));
             b0 = __shfl_sync(0xffffffffu, b0, 0);
             const int64_t at = (int64_t)b0 + __popc(ball & ((1u << l) - 1u));
             if (due) {
@@ -623,20 +606,15 @@ __device__ void predict_select_pass(const State &st, const Records &rec, int64_t
     }
 }
 
-// Table 1 section 8: correct the m listed particles and take their new steps,
-// three lanes per particle in units of kCorrUnit particles per warp; warp w of
+// Table 1 section 8: correct the listed particles q0 .. m - 1 and take their new
+// steps, three lanes per particle in units of kCorrUnit particles per warp; warp w of
 // W takes units w, w + W, ...  low receives the minimum of their new tend.
-__device__ void correct_pass(const State &st, const int32_t *idx, int64_t m, int64_t n, const double *ra,
-                             const double *rj, const double *rs, const double *rn, const StepParams &sp, int32_t *err,
-                             int64_t w, int64_t W, long long &low)
+template <int P, class R>
+__device__ __forceinline__ void correct_pass(const State &st, const int32_t *idx, int64_t q0, int64_t m, int64_t n, const R &res,
+                             const StepParams &sp, int32_t *err, int64_t w, int64_t W, long long &low)
 {
-    const int64_t units = (m + kCorrUnit - 1) / kCorrUnit;
-    for (int64_t u = w; u < units; u += W) {   // warp-uniform
-        if (sp.order == 4)
-            correct_lane<4>(st, idx, ra, rj, rs, rn, sp, m, n, err, u, low);
-        else
-            correct_lane<6>(st, idx, ra, rj, rs, rn, sp, m, n, err, u, low);
-    }
+    for (int64_t q = q0 + w * kCorrUnit; q < m; q += W * kCorrUnit)   // warp-uniform
+        correct_lane<P>(st, idx, res, sp, m, n, err, q, low);
 }
 
 // Next block time: the minimum over the new tend of the corrected particles
@@ -656,11 +634,11 @@ __device__ long long scan_min_pass(const State &st, int64_t n, long long tb, int
     return low;
 }
 
-// One atomicMin per CTA of its threads' minima into sc->tnext_bits.
-__device__ void publish_min(DevScalars *sc, long long low, long long *sh)
+// One atomicMin per CTA of its threads' minima into *tnext_bits.
+__device__ void publish_min(int64_t *tnext_bits, long long low, long long *sh)
 {
     low = block_min_ll(low, sh);
-    if (threadIdx.x == 0 && low != LLONG_MAX) atomicMin((long long *)&sc->tnext_bits, low);
+    if (threadIdx.x == 0 && low != LLONG_MAX) atomicMin((long long *)tnext_bits, low);
 }
 
 }  // namespace
