@@ -310,7 +310,7 @@ struct Mixed {
     // (lane_j == 0) hold out = hi - lo in FP64.  On GB300 an FP64 warp
     // instruction costs ~64 cycles, so the tree stays in FP32 and the widening
     // uses the integer f2d.
-    __device__ static void epilogue(Acc &a, int tpi, int tid, double *red, double (&out)[I][kOut])
+    __device__ static void epilogue(Acc &a, int, int tpi, int tid, double *red, double (&out)[I][kOut])
     {
         const int wspan = tpi < 32 ? tpi : 32;
         for (int off = 1; off < wspan; off <<= 1) {
@@ -375,7 +375,7 @@ struct Mixed {
 struct F64 {
     static constexpr int TJ = kTJF64;
     static constexpr int I = 1;
-    static constexpr int kMinBlocks = 3;
+    static constexpr int kMinBlocks = 2;
     static constexpr int kVariant = 0;
     static constexpr uint32_t kStageBytes = TJ * 80;
     struct ITile {
@@ -423,11 +423,64 @@ struct F64 {
         }
     }
 
+    // Sums of up to kFold64 - 1 pairs a lane and 16 lanes or more an i-particle (small
+    // blocks): the lanes' integer sums are added as integers, and lane c converts
+    // component c.  The FP64 instructions of the general path (36 to fold and 45 in the
+    // tree, 64 cycles each) made a block of one particle of 32768 take 20 us, 15 now.
+    __device__ static void epilogue_small(Acc &a, int pairs, int tpi, int tid, double *red, double (&out)[I][kOut])
+    {
+        constexpr uint32_t kAll = 0xffffffffu;
+        const int warp = tid >> 5, lane = tid & 31, span = tpi < 32 ? tpi : 32, c = lane & (span - 1);
+        int E[3] = {a.E[0], a.E[1], a.E[2]};
+        uint32_t low = a.low;
+        for (int off = 1; off < span; off <<= 1) {
+#pragma unroll
+            for (int g = 0; g < 3; ++g) {
+                const int e = __shfl_xor_sync(kAll, E[g], off);
+                E[g] = e > E[g] ? e : E[g];
+            }
+            const uint32_t l = __shfl_xor_sync(kAll, low, off);
+            low = l < low ? l : low;
+        }
+        p64::align_sums(a, E, pairs * span);
+        for (int off = 1; off < span; off <<= 1) {
+#pragma unroll
+            for (int k = 0; k < 9; ++k) {
+                const int64_t H2 = __shfl_xor_sync(kAll, (long long)a.H[k], off);
+                const uint32_t M2 = __shfl_xor_sync(kAll, a.M[k], off);
+                p64::add_sums(a.H[k], a.M[k], H2, M2);
+            }
+        }
+        int64_t H = a.H[0];
+        uint32_t M = a.M[0];
+#pragma unroll
+        for (int k = 1; k < 9; ++k) {
+            H = c == k ? a.H[k] : H;
+            M = c == k ? a.M[k] : M;
+        }
+        const int e = c < 3 ? a.E[0] : (c < 6 ? a.E[1] : a.E[2]);
+        double v = p64::sum_of(H, M, e, c < 9 ? c : 8);
+        if (low < 0x100000u) v = NAN;
+        if (tpi > 32) {   // two warps an i-particle
+            if (lane < 9) red[warp * kOut + lane] = v;
+            __syncthreads();
+            if (lane < 9) v = red[(warp & ~1) * kOut + lane] + red[(warp | 1) * kOut + lane];
+            __syncthreads();
+        }
+#pragma unroll
+        for (int k = 0; k < 9; ++k) out[0][k] = __shfl_sync(kAll, v, (lane & ~(span - 1)) + k);
+        out[0][9] = 0.0;
+    }
+
     // Sum the tpi lanes sharing an i-particle (fixed xor tree; shared memory
     // across warps for tpi = 64): the leader lanes (lane_j == 0) hold out.  No
     // noise scale (out[k][9] = 0): the FP64 path needs no noise floor.
-    __device__ static void epilogue(Acc &a, int tpi, int tid, double *red, double (&out)[I][kOut])
+    __device__ static void epilogue(Acc &a, int pairs, int tpi, int tid, double *red, double (&out)[I][kOut])
     {
+        if (tpi >= 16 && pairs < p64::kFold64) {   // the same in every thread of the CTA
+            epilogue_small(a, pairs, tpi, tid, red, out);
+            return;
+        }
         p64::finish(a);
 #pragma unroll
         for (int k = 0; k < I; ++k) {
@@ -581,7 +634,7 @@ __device__ bool eval_items(const EvalArgs &args, int64_t m, const Plan &pl, unsi
         seq += (uint32_t)nt;
 
         double out[P::I][kOut];
-        P::epilogue(acc, tpi, tid, red, out);
+        P::epilogue(acc, nt * (P::TJ / tpi), tpi, tid, red, out);
         if (!batch && args.direct_b1 && pl.b == 1) {   // no j-split: these are the results
             if (lane_j == 0) {
 #pragma unroll

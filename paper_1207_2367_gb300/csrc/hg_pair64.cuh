@@ -57,6 +57,7 @@ constexpr int kFold64 = 32;               // pairs between additions to the FP64
 // it moves less often.
 constexpr int kBitsQ = 59, kSlack = 2;
 constexpr int kExpNone = -(1 << 28);      // exponent of an empty sum
+static_assert(kFold64 == 32, "the room of align_sums");
 
 struct Limbs {
     int32_t h, l;
@@ -410,6 +411,29 @@ HG_P64 void fold_fp64(Sums &a)
         a.H[c] = 0;
     }
     a.cnt = 0;
+}
+
+// Component c of the integer sums alone.
+HG_P64 double sum_of(int64_t H, uint32_t M, int E, int c)
+{
+    const int e = E - unit(c / 3);
+    return add_scaled(add_scaled(0.0, H, e), (int64_t)(uint64_t)M, e - 32);
+}
+
+// Sums of lanes that together took `all` pairs, the same number each and none folded
+// yet: moves this lane's to the exponents E, with room for the total.
+HG_P64 void align_sums(Sums &a, const int (&E)[3], int all)
+{
+    const int room = all > kFold64 ? 32 - clz32((uint32_t)(all - 1)) - 5 : 0;
+#pragma unroll
+    for (int c = 0; c < 9; ++c) shift_sum(a.H[c], a.M[c], E[c / 3] + room - a.E[c / 3]);
+    for (int g = 0; g < 3; ++g) a.E[g] = E[g] + room;
+}
+HG_P64 void add_sums(int64_t &H, uint32_t &M, int64_t H2, uint32_t M2)
+{
+    const uint64_t m = (uint64_t)M + M2;
+    M = (uint32_t)m;
+    H += H2 + (int64_t)(m >> 32);
 }
 
 HG_P64 void count_pair(Sums &a)
