@@ -151,6 +151,19 @@ bool is_device_ptr(const void *p)
     return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
+// Plain memory of the context's GPU, aligned for T: kernels may write it.
+template <class T>
+bool is_own_memory(const hg_ctx *c, const T *p)
+{
+    cudaPointerAttributes a;
+    if (!p || ((uintptr_t)p & (sizeof(T) - 1)) != 0) return false;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return a.type == cudaMemoryTypeDevice && a.device == c->device;
+}
+
 template <class T>
 T *dalloc(hg_ctx *c, int64_t count)
 {
@@ -235,8 +248,8 @@ cudaError_t batch_plan(hg_ctx *c, const int64_t *m_dev, int64_t m_host, cudaStre
     return launch_batch_plan(c->d_idx, m_dev, m_host, c->bv, c->pp, m_dev ? c->d_sc : nullptr, s);
 }
 
-// Evaluation of the list in d_idx (host-known size m) into ra/rj/rs.
-int run_eval_host_m(hg_ctx *c, int64_t m)
+// Evaluation of the list in d_idx (host-known size m) into ra/rj/rs (and out).
+int run_eval_host_m(hg_ctx *c, int64_t m, const EvalOut &out = EvalOut{})
 {
     EvalArgs a = eval_args(c, nullptr, m);
     if (c->bv.nc > 0) {
@@ -244,7 +257,7 @@ int run_eval_host_m(hg_ctx *c, int64_t m)
         c->kernels += 1;
     }
     HG_CUDA(c, launch_eval(c->mixed, a, c->num_sms, c->stream));
-    HG_CUDA(c, launch_reduce(a, c->ra, c->rj, c->rs, 2 * c->num_sms, c->stream));
+    HG_CUDA(c, launch_reduce(a, c->ra, c->rj, c->rs, out, 2 * c->num_sms, c->stream));
     c->kernels += 2;
     return HG_OK;
 }
@@ -887,8 +900,11 @@ int hg_next_block(hg_ctx *c, double *t_next, int32_t *idx, int64_t cap, int64_t 
     const CallRange range_("hg_next_block");
     if (!c) return HG_EINVAL;
     if (const int rb = sync_bound(c)) return rb;
-    HG_CUDA(c, launch_next_block(c->st, c->n, c->nb_part, c->nb_cnt, c->nb_off, c->d_idx, c->d_sc, c->stream));
-    c->kernels += 3;
+    // A device array that holds any block takes the list from the kernels.
+    const bool direct = cap >= c->n && is_own_memory(c, idx);
+    HG_CUDA(c, launch_next_block(c->st, c->n, c->nb_part, c->nb_cnt, c->nb_off, c->d_idx, direct ? idx : nullptr,
+                                 c->d_sc, c->stream));
+    c->kernels += next_block_kernels(c->n);
     int rc = sync_scalars(c);
     if (rc) return rc;
     const int64_t m = c->h_sc->m;
@@ -896,7 +912,7 @@ int hg_next_block(hg_ctx *c, double *t_next, int32_t *idx, int64_t cap, int64_t 
     c->cur_m = m;
     if (t_next) *t_next = c->h_sc->t_cur;
     if (m_out) *m_out = m;
-    if (idx) {
+    if (idx && !direct) {
         if (cap < m) return fail(c, HG_EINVAL, "idx capacity smaller than the block");
         HG_CUDA(c, cudaMemcpyAsync(idx, c->d_idx, m * sizeof(int32_t), cudaMemcpyDefault, c->stream));
         HG_CUDA(c, cudaStreamSynchronize(c->stream));
@@ -946,12 +962,20 @@ int hg_evaluate(hg_ctx *c, const int32_t *idx, int64_t m, double *acc, double *j
         drop_graphs(c);   // they captured the old list pointer
     }
     if (m > 0) {
-        int rc = run_eval_host_m(c, m);
-        if (rc) return rc;
+        // Device arrays take the results from the reduction kernel, unless they overlap
+        // (then copied one after the other).
         double *outs[3] = {acc, jerk, snap};
+        EvalOut direct;
+        for (int k = 0; k < 3; ++k)
+            if (is_own_memory(c, outs[k])) direct.p[k] = outs[k];
+        for (int k = 0; k < 3; ++k)
+            for (int j = 0; j < k; ++j)
+                if (outs[j] && outs[k] && outs[k] < outs[j] + 3 * m && outs[j] < outs[k] + 3 * m) direct = EvalOut{};
+        int rc = run_eval_host_m(c, m, direct);
+        if (rc) return rc;
         const double *res[3] = {c->ra, c->rj, c->rs};
         for (int k = 0; k < 3; ++k)
-            if (outs[k])
+            if (outs[k] && !direct.p[k])
                 HG_CUDA(c, cudaMemcpyAsync(outs[k], res[k], 3 * m * sizeof(double), cudaMemcpyDefault, c->stream));
     }
     int rc = sync_scalars(c);

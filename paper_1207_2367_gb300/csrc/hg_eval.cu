@@ -691,8 +691,8 @@ __global__ void __launch_bounds__(kEvalThreads, P::kMinBlocks) k_eval(const Eval
 // Table 1 section 4: sum the b j-chunk partials of every listed particle in
 // chunk order and scatter them to acc/jerk/snap [m][3] (and the noise scale to
 // args.rn [m] when it is set).
-__device__ __forceinline__ void put_result(const EvalArgs &a, double *ra, double *rj, double *rs, int64_t q, int c,
-                                           double v)
+__device__ __forceinline__ void put_result(const EvalArgs &a, double *ra, double *rj, double *rs, const EvalOut &out,
+                                           int64_t q, int c, double v)
 {
     if (c == 9) {
         if (a.rn) a.rn[q] = v;
@@ -700,15 +700,24 @@ __device__ __forceinline__ void put_result(const EvalArgs &a, double *ra, double
     }
     double *dst = c < 3 ? ra : (c < 6 ? rj : rs);
     dst[q * 3 + (c % 3)] = v;
+    double *o = out.p[c / 3];
+    if (o) o[q * 3 + (c % 3)] = v;
 }
 
 // The reduction's values taken by global thread g of G threads (grid-stride):
 // the body of k_reduce.
 // Each (particle, value) sum has a fixed order whichever thread takes it.
 __device__ void reduce_values(const EvalArgs &args, int64_t m, const Plan &pl, double *ra, double *rj, double *rs,
-                              int64_t g, int64_t G)
+                              const EvalOut &out, int64_t g, int64_t G)
 {
-    if (args.bv.nc == 0 && args.direct_b1 && pl.b == 1) return;   // the evaluation wrote the results
+    if (args.bv.nc == 0 && args.direct_b1 && pl.b == 1) {   // the evaluation wrote the results
+        const double *res[3] = {ra, rj, rs};
+#pragma unroll
+        for (int d = 0; d < 3; ++d)
+            if (out.p[d])
+                for (int64_t e = g; e < 3 * m; e += G) out.p[d][e] = __ldcg(res[d] + e);
+        return;
+    }
     const int64_t total = m * kOut;
     if (args.bv.nc > 0) {
         // Clusters: the chunks of position q are rows part_off[c] + s * m_c + (q - a_off[c]).
@@ -725,7 +734,7 @@ __device__ void reduce_values(const EvalArgs &args, int64_t m, const Plan &pl, d
             if (!in_bounds(row0 >= 0 && row0 + (int64_t)(b - 1) * mc < args.pcap, args.err)) continue;
             double s = 0.0;
             for (int sp = 0; sp < b; ++sp) s += __ldcg(args.partial + (row0 + (int64_t)sp * mc) * kOut + cv);
-            put_result(args, ra, rj, rs, q, cv, s);
+            put_result(args, ra, rj, rs, out, q, cv, s);
         }
         return;
     }
@@ -737,7 +746,7 @@ __device__ void reduce_values(const EvalArgs &args, int64_t m, const Plan &pl, d
             const int c = (int)(e - q * kOut);
             double s = 0.0;
             for (int sp = 0; sp < pl.b; ++sp) s += __ldcg(args.partial + ((int64_t)sp * m + q) * kOut + c);
-            put_result(args, ra, rj, rs, q, c, s);
+            put_result(args, ra, rj, rs, out, q, c, s);
         }
     } else {
         // Many chunks (small blocks): one warp per (particle, value); lane l
@@ -754,17 +763,17 @@ __device__ void reduce_values(const EvalArgs &args, int64_t m, const Plan &pl, d
             double s = 0.0;
             for (int sp = lane; sp < pl.b; sp += 32) s += __ldcg(args.partial + ((int64_t)sp * m + q) * kOut + c);
             for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-            if (lane == 0) put_result(args, ra, rj, rs, q, c, s);
+            if (lane == 0) put_result(args, ra, rj, rs, out, q, c, s);
         }
     }
 }
 
-__global__ void k_reduce(const EvalArgs args, double *ra, double *rj, double *rs)
+__global__ void k_reduce(const EvalArgs args, double *ra, double *rj, double *rs, const EvalOut out)
 {
     const int64_t m = args.m_host;   // explicit calls; graph steps sum in the correction
     if (m <= 0) return;
     const Plan pl = args.plan_host;   // clusters: the work list instead
-    reduce_values(args, m, pl, ra, rj, rs, blockIdx.x * (int64_t)blockDim.x + threadIdx.x,
+    reduce_values(args, m, pl, ra, rj, rs, out, blockIdx.x * (int64_t)blockDim.x + threadIdx.x,
                   (int64_t)gridDim.x * blockDim.x);
 }
 
@@ -854,9 +863,10 @@ cudaError_t launch_plan_one(Plan *plan, const int64_t *m_dev, const PlanParams &
     return cudaGetLastError();
 }
 
-cudaError_t launch_reduce(const EvalArgs &args, double *ra, double *rj, double *rs, int grid, cudaStream_t st)
+cudaError_t launch_reduce(const EvalArgs &args, double *ra, double *rj, double *rs, const EvalOut &out, int grid,
+                          cudaStream_t st)
 {
-    k_reduce<<<grid, 256, 0, st>>>(args, ra, rj, rs);
+    k_reduce<<<grid, 256, 0, st>>>(args, ra, rj, rs, out);
     return cudaGetLastError();
 }
 

@@ -306,6 +306,11 @@ struct EvalArgs {
     double *rn = nullptr;              // [m] noise scale (nullptr: not written)
 };
 
+// Second copies of the results, [m][3] each, or nullptr (the caller's device arrays).
+struct EvalOut {
+    double *p[3] = {nullptr, nullptr, nullptr};
+};
+
 // Planner inputs of one precision (hg_eval.cu): tiles, tile size, i per thread,
 // overhead constants and the persistent grid of the evaluation kernel.
 PlanParams plan_params(bool mixed, int64_t npad, int num_sms, int64_t pcap, int tpi_force, int b_force);
@@ -324,8 +329,9 @@ cudaError_t launch_plan_table(Plan *tab, int64_t n, const PlanParams &pq, cudaSt
 cudaError_t launch_plan_one(Plan *plan, const int64_t *m_dev, const PlanParams &pq, cudaStream_t st);
 // Sums the b partials of each listed particle into res_{a,j,s} [m][3] and, when
 // args.rn is set, the noise scale into args.rn [m] (grid-stride: grid CTAs of
-// 256 threads, a few per SM).
-cudaError_t launch_reduce(const EvalArgs &args, double *ra, double *rj, double *rs, int grid, cudaStream_t st);
+// 256 threads, a few per SM); the results also into out.
+cudaError_t launch_reduce(const EvalArgs &args, double *ra, double *rj, double *rs, const EvalOut &out, int grid,
+                          cudaStream_t st);
 
 // Bit patterns of IEEE-754 values (host and device).
 __host__ __device__ __forceinline__ unsigned long long bits_of(double x)

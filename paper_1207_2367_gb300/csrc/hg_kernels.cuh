@@ -19,9 +19,11 @@ struct StepParams {
 constexpr int64_t kNBChunk = 2048;   // particles per CTA in the next-block passes
 
 int nb_grid(int64_t n);
-// part, cnt, off: nb_grid(n) entries each.
+// part, cnt, off: nb_grid(n) entries each.  The list goes to idx and, unless it is
+// nullptr, to out (n entries each).
 cudaError_t launch_next_block(const State &st, int64_t n, double *part, int32_t *cnt, int32_t *off, int32_t *idx,
-                              DevScalars *sc, cudaStream_t s);
+                              int32_t *out, DevScalars *sc, cudaStream_t s);
+int next_block_kernels(int64_t n);   // how many it launches
 // Graph steps of clusters: the list of the particles due at sc->tnext_bits[par] (kept by
 // launch_reduce_correct), ascending, and the due particles of each cluster in bv.act.
 cudaError_t launch_select_clusters(const State &st, int64_t n, int32_t *cnt, int32_t *off, int32_t *idx,

@@ -233,7 +233,7 @@ extern "C" int hg_evaluate_static(int64_t n, const double *mass, const double *p
     a.err = err;
     a.direct_b1 = 0;        // partials summed by k_reduce
     if (cudaGetLastError() != cudaSuccess || launch_eval(mixed, a, slot->sms, st) != cudaSuccess ||
-        launch_reduce(a, acc, jerk, snap, 2 * slot->sms, st) != cudaSuccess) {
+        launch_reduce(a, acc, jerk, snap, EvalOut{}, 2 * slot->sms, st) != cudaSuccess) {
         set_call_error("launch failed");
         return HG_ECUDA;
     }
