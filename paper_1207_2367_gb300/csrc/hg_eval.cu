@@ -673,6 +673,8 @@ __global__ void __launch_bounds__(kEvalThreads, P::kMinBlocks) k_eval(const Eval
     extern __shared__ __align__(128) unsigned char smem[];
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + kStages * P::kStageBytes);
     double *red = reinterpret_cast<double *>(bars + kStages);
+    wait_for_previous();
+    let_next_start();
     const int64_t m = args.m_dev ? *args.m_dev : args.m_host;
     if (m <= 0) return;
     const Plan pl = args.plan_dev ? args.plan_dev[(m - 1) * args.plan_stride] : args.plan_host;
@@ -813,11 +815,8 @@ namespace {
 template <class P>
 cudaError_t launch_one(const EvalArgs &args, int grid, cudaStream_t st)
 {
-    if (args.guard)
-        k_eval<P, true><<<grid, kEvalThreads, smem_bytes<P>(), st>>>(args);
-    else
-        k_eval<P, false><<<grid, kEvalThreads, smem_bytes<P>(), st>>>(args);
-    return cudaGetLastError();
+    return launch_dependent(args.guard ? k_eval<P, true> : k_eval<P, false>, grid, kEvalThreads, smem_bytes<P>(), st,
+                            args);
 }
 
 template <class P>

@@ -286,6 +286,7 @@ template <bool MIXED>
 __global__ void __launch_bounds__(kSelThreads) k_predict_select(const State st, const Records rec, int64_t n,
                                                                 int64_t npad, int32_t *idx, DevScalars *sc, int par)
 {
+    wait_for_previous();
     const long long tn = *((volatile long long *)&sc->tnext_bits[par]);
     const double t_next = __longlong_as_double(tn);
     const bool take = t_next <= *((volatile double *)&sc->t_stop);
@@ -384,6 +385,7 @@ __global__ void __launch_bounds__(kStepThreads) k_reduce_correct(State st, const
 {
     __shared__ long long sh[32];
     __shared__ double rows[kStepChunk * kOut];
+    wait_for_previous();
     const int64_t m = BATCH ? *((volatile int64_t *)&sc->m) : (int64_t)*((volatile unsigned long long *)&sc->slot[par]);
     if (m <= 0) return;
     const int b = BATCH ? 0 : plan[(m - 1) * plan_stride].b;   // clusters have their own
@@ -1006,11 +1008,8 @@ cudaError_t launch_predict_select(bool mixed, const State &st, const Records &re
                                   int32_t *idx, DevScalars *sc, int par, cudaStream_t s)
 {
     const int g = grid_for(npad, kSelThreads, 1 << 20);
-    if (mixed)
-        k_predict_select<true><<<g, kSelThreads, 0, s>>>(st, rec, n, npad, idx, sc, par);
-    else
-        k_predict_select<false><<<g, kSelThreads, 0, s>>>(st, rec, n, npad, idx, sc, par);
-    return cudaGetLastError();
+    return launch_dependent(mixed ? k_predict_select<true> : k_predict_select<false>, g, kSelThreads, 0, s, st, rec, n,
+                            npad, idx, sc, par);
 }
 
 cudaError_t launch_swap_entries(DevScalars *sc, cudaStream_t s)
@@ -1066,14 +1065,11 @@ cudaError_t launch_reduce_correct(const State &st, const int32_t *idx, int64_t n
                                   const StepParams &sp, DevScalars *sc, int par, int grid, cudaStream_t s)
 {
     auto launch = [&](auto kernel) {
-        kernel<<<grid, kStepThreads, 0, s>>>(st, idx, n, a.partial, a.pcap, ResultArrays{{a.ra, a.rj, a.rs}, a.rn},
-                                             a.bv, a.plan_dev, a.plan_stride, sp, sc, par);
+        return launch_dependent(kernel, grid, kStepThreads, 0, s, st, idx, n, (const double *)a.partial, a.pcap,
+                                ResultArrays{{a.ra, a.rj, a.rs}, a.rn}, a.bv, a.plan_dev, a.plan_stride, sp, sc, par);
     };
-    if (a.bv.nc > 0)
-        sp.order == 4 ? launch(k_reduce_correct<4, true>) : launch(k_reduce_correct<6, true>);
-    else
-        sp.order == 4 ? launch(k_reduce_correct<4, false>) : launch(k_reduce_correct<6, false>);
-    return cudaGetLastError();
+    if (a.bv.nc > 0) return sp.order == 4 ? launch(k_reduce_correct<4, true>) : launch(k_reduce_correct<6, true>);
+    return sp.order == 4 ? launch(k_reduce_correct<4, false>) : launch(k_reduce_correct<6, false>);
 }
 
 int energy_splits(int64_t n, int num_sms)
