@@ -329,7 +329,9 @@ def roofline(hg, inter, prof, mixed, mhz, kind, traffic=None, measured=None):
            "flops_per_interaction_rsqrt_as_4": flops + 4,
            "paper_flops_per_interaction": PAPER_FLOPS,
            "peak_note": ((f"FP32 FMA pipe: {NUM_SMS} SMs x 128 lanes x 2 flops" if mixed else
-                          f"FP64 pipe: {NUM_SMS} SMs x 2 DFMA x 2 flops") + f" x {mhz:.0f} MHz ({kind} max clock)"),
+                          f"FP64 pipe: {NUM_SMS} SMs x 2 DFMA x 2 flops; all but the differences of a pair run as "
+                          f"64-bit fixed point on the integer pipes, so the share may exceed 1,")
+                         + f" x {mhz:.0f} MHz ({kind} max clock)"),
            "eval_share_of_step": eval_s / (sum(prof["ms"].values()) / 1e3) if prof["ms"] else None}
     if measured:
         mp = max(measured.get("f32", 0.0), measured.get("f32x2", 0.0)) if mixed else measured.get("f64", 0.0)

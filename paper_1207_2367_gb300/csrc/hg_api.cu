@@ -28,7 +28,8 @@ struct hg_ctx {
     double eps = 0.0, eta = 0.0;
     hg_opts opts{};
     int device = 0, num_sms = 0;
-    cudaStream_t stream = nullptr, cap_stream = nullptr;
+    cudaStream_t stream = nullptr, cap_stream = nullptr, cap_side = nullptr;
+    cudaEvent_t ev_fork[2] = {nullptr, nullptr};   // of the side branch in captured cluster steps
     bool own_stream = false;
     State st{}, st2{};
     State own{};          // the context's own state arrays (st points at the caller's when bound)
@@ -320,7 +321,13 @@ int enqueue_block_step(hg_ctx *c, cudaStream_t s, int par, const cudaEvent_t *ev
     const bool batch = c->bv.nc > 0;
     if (ev) HG_CUDA(c, record_external(ev[0], s));
     if (batch) {
-        HG_CUDA(c, launch_select_clusters(c->st, c->n, c->nb_cnt, c->nb_off, c->d_idx, c->d_sc, par, c->bv, s));
+        // The list, which only the evaluation and the correction read, is made beside
+        // the plan and the prediction (5.3 us off the step's chain).
+        HG_CUDA(c, launch_count_due(c->st, c->n, c->nb_cnt, c->nb_off, c->d_sc, par, c->bv, s));
+        HG_CUDA(c, cudaEventRecord(c->ev_fork[0], s));
+        HG_CUDA(c, cudaStreamWaitEvent(c->cap_side, c->ev_fork[0], 0));
+        HG_CUDA(c, launch_list_due(c->st, c->n, c->nb_off, c->d_idx, c->d_sc, c->cap_side));
+        HG_CUDA(c, cudaEventRecord(c->ev_fork[1], c->cap_side));
         HG_CUDA(c, batch_plan(c, &c->d_sc->m, 0, s));
     }
     if (ev) HG_CUDA(c, record_external(ev[1], s));
@@ -332,6 +339,7 @@ int enqueue_block_step(hg_ctx *c, cudaStream_t s, int par, const cudaEvent_t *ev
     const int64_t *m_dev = batch ? &c->d_sc->m : reinterpret_cast<const int64_t *>(&c->d_sc->slot[par]);
     EvalArgs a = eval_args(c, m_dev, 0);
     if (!batch && c->n > kPlanTable) HG_CUDA(c, launch_plan_one(c->plan_tab, m_dev, c->pp, s));
+    if (batch) HG_CUDA(c, cudaStreamWaitEvent(s, c->ev_fork[1], 0));
     HG_CUDA(c, launch_eval(c->mixed, a, c->num_sms, s));
     if (ev) HG_CUDA(c, record_external(ev[3], s));
     if (ev) HG_CUDA(c, record_external(ev[4], s));
@@ -457,6 +465,9 @@ void release(hg_ctx *c)
     if (c->h_flags) cudaFreeHost(c->h_flags);
     for (cudaEvent_t e : c->ev_flags)
         if (e) cudaEventDestroy(e);
+    for (cudaEvent_t e : c->ev_fork)
+        if (e) cudaEventDestroy(e);
+    if (c->cap_side) cudaStreamDestroy(c->cap_side);
     if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
     if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);
     cudaGetLastError();
@@ -477,6 +488,10 @@ int init_impl(hg_ctx *c, const double *mass, const double *pos, const double *ve
         c->own_stream = true;
     }
     HG_CUDA(c, cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking));
+    if (!c->cl_off_host.empty()) {
+        HG_CUDA(c, cudaStreamCreateWithFlags(&c->cap_side, cudaStreamNonBlocking));
+        for (cudaEvent_t &e : c->ev_fork) HG_CUDA(c, cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+    }
     HG_CUDA(c, cudaMallocHost(reinterpret_cast<void **>(&c->h_sc), sizeof(DevScalars)));
     HG_CUDA(c, cudaMallocHost(reinterpret_cast<void **>(&c->h_stage), 4 * sizeof(double)));
     HG_CUDA(c, cudaMallocHost(reinterpret_cast<void **>(&c->h_flags), 4 * sizeof(int32_t)));

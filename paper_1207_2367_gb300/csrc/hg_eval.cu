@@ -815,6 +815,13 @@ namespace {
 template <class P>
 cudaError_t launch_one(const EvalArgs &args, int grid, cudaStream_t st)
 {
+    if (args.bv.nc > 0) {   // follows two branches of the step's graph: an ordinary launch
+        if (args.guard)
+            k_eval<P, true><<<grid, kEvalThreads, smem_bytes<P>(), st>>>(args);
+        else
+            k_eval<P, false><<<grid, kEvalThreads, smem_bytes<P>(), st>>>(args);
+        return cudaGetLastError();
+    }
     return launch_dependent(args.guard ? k_eval<P, true> : k_eval<P, false>, grid, kEvalThreads, smem_bytes<P>(), st,
                             args);
 }

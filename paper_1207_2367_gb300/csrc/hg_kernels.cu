@@ -963,12 +963,18 @@ cudaError_t launch_next_block(const State &st, int64_t n, double *part, int32_t 
     return cudaGetLastError();
 }
 
-cudaError_t launch_select_clusters(const State &st, int64_t n, int32_t *cnt, int32_t *off, int32_t *idx,
-                                   DevScalars *sc, int par, const BatchView &bv, cudaStream_t s)
+cudaError_t launch_count_due(const State &st, int64_t n, int32_t *cnt, int32_t *off, DevScalars *sc, int par,
+                             const BatchView &bv, cudaStream_t s)
 {
     const int g = nb_grid(n);
     k_nb_count<<<g, kNBThreads, 0, s>>>(st.tend, n, kNBChunk, cnt, off, g, sc, 1, par, bv.cl_of, bv.act);
-    k_nb_scatter<<<g, kNBThreads, 0, s>>>(st.tend, n, kNBChunk, off, idx, nullptr, sc);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_list_due(const State &st, int64_t n, const int32_t *off, int32_t *idx, DevScalars *sc,
+                            cudaStream_t s)
+{
+    k_nb_scatter<<<nb_grid(n), kNBThreads, 0, s>>>(st.tend, n, kNBChunk, off, idx, nullptr, sc);
     return cudaGetLastError();
 }
 

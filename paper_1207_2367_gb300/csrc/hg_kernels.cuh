@@ -24,10 +24,13 @@ int nb_grid(int64_t n);
 cudaError_t launch_next_block(const State &st, int64_t n, double *part, int32_t *cnt, int32_t *off, int32_t *idx,
                               int32_t *out, DevScalars *sc, cudaStream_t s);
 int next_block_kernels(int64_t n);   // how many it launches
-// Graph steps of clusters: the list of the particles due at sc->tnext_bits[par] (kept by
-// launch_reduce_correct), ascending, and the due particles of each cluster in bv.act.
-cudaError_t launch_select_clusters(const State &st, int64_t n, int32_t *cnt, int32_t *off, int32_t *idx,
-                                   DevScalars *sc, int par, const BatchView &bv, cudaStream_t s);
+// Graph steps of clusters: how many particles are due at sc->tnext_bits[par] (kept by
+// launch_reduce_correct), in each cluster (bv.act) and chunk (cnt, off); then their
+// list, ascending.
+cudaError_t launch_count_due(const State &st, int64_t n, int32_t *cnt, int32_t *off, DevScalars *sc, int par,
+                             const BatchView &bv, cudaStream_t s);
+cudaError_t launch_list_due(const State &st, int64_t n, const int32_t *off, int32_t *idx, DevScalars *sc,
+                            cudaStream_t s);
 // Pass 1 alone: sc->tnext_bits[0] = bits of min_i tend_i.
 cudaError_t launch_next_min(const State &st, int64_t n, double *part, DevScalars *sc, cudaStream_t s);
 // One system, graph-replayed block steps: block selection fused into the
