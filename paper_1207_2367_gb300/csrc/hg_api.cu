@@ -64,6 +64,8 @@ struct hg_ctx {
     int64_t eval_m = -1;    // size of the last hg_evaluate (-1: none pending)
     double eval_t = NAN;
     std::vector<void *> dev_allocs;
+    char *slab = nullptr;        // the newest shared block of device memory and what is left of it
+    size_t slab_left = 0;
     std::string err;
 };
 
@@ -168,15 +170,28 @@ bool is_own_memory(const hg_ctx *c, const T *p)
 template <class T>
 T *dalloc(hg_ctx *c, int64_t count)
 {
-    void *p = nullptr;
     if (count < 1) count = 1;
     if (fault_point(HG_FAULT_ALLOC)) return nullptr;
-    if (cudaMalloc(&p, (size_t)count * sizeof(T)) != cudaSuccess) {
-        cudaGetLastError();
-        return nullptr;
+    // Arrays share blocks of 512 B a particle (256 KB to 64 MB), the larger half of them
+    // have their own: a context has ~45 arrays, and a cudaMalloc each was most of hg_init.
+    const size_t bytes = ((size_t)count * sizeof(T) + 255) & ~(size_t)255;
+    const size_t block = std::min<size_t>(std::max<size_t>((size_t)c->n * 512, (size_t)256 << 10), (size_t)64 << 20);
+    const bool own = bytes > block / 2;
+    if (own || bytes > c->slab_left) {
+        void *p = nullptr;
+        if (cudaMalloc(&p, own ? bytes : block) != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        c->dev_allocs.push_back(p);
+        if (own) return static_cast<T *>(p);
+        c->slab = static_cast<char *>(p);
+        c->slab_left = block;
     }
-    c->dev_allocs.push_back(p);
-    return static_cast<T *>(p);
+    T *p = reinterpret_cast<T *>(c->slab);
+    c->slab += bytes;
+    c->slab_left -= bytes;
+    return p;
 }
 
 bool alloc_state(hg_ctx *c, State &s)
@@ -585,14 +600,17 @@ int init_impl(hg_ctx *c, const double *mass, const double *pos, const double *ve
     c->xe = dalloc<double>(c, 3 * n);
     c->ve = dalloc<double>(c, 3 * n);
     c->e_splits = energy_splits(n, c->num_sms);
-    c->phi_part = dalloc<double>(c, (int64_t)c->e_splits * n);
+    // The energy's per-split potentials use the evaluation's partial-sum buffer (free
+    // between calls; pcap >= n rows of kOut).
+    c->e_splits = (int)std::min<int64_t>(c->e_splits, (int64_t)kOut * pcap / n);
+    c->phi_part = c->partial;
     c->e_g2 = (int)((n + 255) / 256 < 1024 ? (n + 255) / 256 : 1024);
     c->e_part = dalloc<double>(c, 2 * c->e_g2);
     c->e_out = dalloc<double>(c, 2);
     c->l_part = dalloc<double>(c, 3 * c->e_g2);
     c->l_out = dalloc<double>(c, 3);
     ok = ok && c->d_idx && c->d_idx2 && c->nb_part && c->nb_cnt && c->nb_off && c->d_sc && c->plan_tab && c->partial && c->ra &&
-         c->rj && c->rs && c->rn && c->xe && c->ve && c->phi_part && c->e_part && c->e_out && c->l_part && c->l_out;
+         c->rj && c->rs && c->rn && c->xe && c->ve && c->e_part && c->e_out && c->l_part && c->l_out;
     if (!ok) return fail(c, HG_ENOMEM, "device allocation failed");
 
     HG_CUDA(c, eval_setup(c->device));
