@@ -53,7 +53,10 @@ struct hg_ctx {
     double *xe = nullptr, *ve = nullptr, *phi_part = nullptr, *e_part = nullptr, *e_out = nullptr;
     double *l_part = nullptr, *l_out = nullptr;   // angular momentum: 3 partials per CTA, result
     int e_splits = 0, e_g2 = 0;
-    cudaGraphExec_t g_one = nullptr, g_many = nullptr;
+    // Graphs of one and of graph_steps block steps, by the entry of the selection's
+    // scalars they start from, and the entry the next step starts from.
+    cudaGraphExec_t g_one[2] = {nullptr, nullptr}, g_many[2] = {nullptr, nullptr};
+    int par = 0;
     int64_t kernels = 0;            // kernel launches issued (graph replays count every node)
     std::vector<cudaEvent_t> ev_one, ev_many;   // profile: 6 events per captured block step
     double prof_ms[5] = {0, 0, 0, 0, 0};
@@ -382,11 +385,12 @@ int ensure_tnext(hg_ctx *c)
     if (c->tnext_valid) return HG_OK;
     HG_CUDA(c, launch_next_min(c->st, c->n, c->nb_part, c->d_sc, c->stream));
     c->kernels += 1;
+    c->par = 0;
     c->tnext_valid = true;
     return HG_OK;
 }
 
-int capture(hg_ctx *c, int steps, cudaGraphExec_t *out, std::vector<cudaEvent_t> &ev)
+int capture(hg_ctx *c, int steps, int par, cudaGraphExec_t *out, std::vector<cudaEvent_t> &ev)
 {
     cudaGraph_t g = nullptr;
     if (c->opts.profile && ev.empty()) {
@@ -396,10 +400,7 @@ int capture(hg_ctx *c, int steps, cudaGraphExec_t *out, std::vector<cudaEvent_t>
     HG_CUDA(c, cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal));
     int rc = HG_OK;
     for (int k = 0; k < steps && rc == HG_OK; ++k)
-        rc = enqueue_block_step(c, c->cap_stream, k & 1, c->opts.profile ? &ev[(size_t)k * 6] : nullptr);
-    // Every graph starts from entry 0: an odd number of steps has left the state in entry 1.
-    if (rc == HG_OK && (steps & 1) && launch_swap_entries(c->d_sc, c->cap_stream) != cudaSuccess)
-        rc = fail(c, HG_ECUDA, "graph capture: launch failed");
+        rc = enqueue_block_step(c, c->cap_stream, (par + k) & 1, c->opts.profile ? &ev[(size_t)k * 6] : nullptr);
     cudaError_t e = cudaStreamEndCapture(c->cap_stream, &g);
     if (rc != HG_OK) {
         if (g) cudaGraphDestroy(g);
@@ -420,17 +421,24 @@ int ensure_graphs(hg_ctx *c)
         c->kernels += 1;
         c->plan_tab_valid = true;
     }
-    if (!c->g_one) rc = capture(c, 1, &c->g_one, c->ev_one);
-    if (rc == HG_OK && !c->g_many) rc = capture(c, c->opts.graph_steps, &c->g_many, c->ev_many);
+    if (!c->g_one[c->par]) rc = capture(c, 1, c->par, &c->g_one[c->par], c->ev_one);
+    if (rc == HG_OK && !c->g_many[c->par])
+        rc = capture(c, c->opts.graph_steps, c->par, &c->g_many[c->par], c->ev_many);
     return rc;
 }
 
 // Launch one captured graph; with profiling, wait for it and add its section times.
 int replay(hg_ctx *c, bool many)
 {
-    HG_CUDA(c, cudaGraphLaunch(many ? c->g_many : c->g_one, c->stream));
     const int steps = many ? c->opts.graph_steps : 1;
-    c->kernels += (int64_t)step_kernels(c) * steps + (steps & 1);
+    cudaGraphExec_t &g = many ? c->g_many[c->par] : c->g_one[c->par];
+    if (!g) {   // an odd number of steps came before
+        const int rc = capture(c, steps, c->par, &g, many ? c->ev_many : c->ev_one);
+        if (rc) return rc;
+    }
+    HG_CUDA(c, cudaGraphLaunch(g, c->stream));
+    c->par ^= steps & 1;
+    c->kernels += (int64_t)step_kernels(c) * steps;
     if (!c->opts.profile) return HG_OK;
     HG_CUDA(c, cudaStreamSynchronize(c->stream));
     const std::vector<cudaEvent_t> &ev = many ? c->ev_many : c->ev_one;
@@ -448,14 +456,11 @@ int replay(hg_ctx *c, bool many)
 // inputs): drop them when those change; they are captured again on next use.
 void drop_graphs(hg_ctx *c)
 {
-    if (c->g_one) {
-        cudaGraphExecDestroy(c->g_one);
-        c->g_one = nullptr;
-    }
-    if (c->g_many) {
-        cudaGraphExecDestroy(c->g_many);
-        c->g_many = nullptr;
-    }
+    for (cudaGraphExec_t *g : {&c->g_one[0], &c->g_one[1], &c->g_many[0], &c->g_many[1]})
+        if (*g) {
+            cudaGraphExecDestroy(*g);
+            *g = nullptr;
+        }
 }
 
 void invalidate(hg_ctx *c)
@@ -470,8 +475,7 @@ void release(hg_ctx *c)
 {
     if (!c) return;
     if (c->stream) cudaStreamSynchronize(c->stream);
-    if (c->g_one) cudaGraphExecDestroy(c->g_one);
-    if (c->g_many) cudaGraphExecDestroy(c->g_many);
+    drop_graphs(c);
     for (cudaEvent_t e : c->ev_one) cudaEventDestroy(e);
     for (cudaEvent_t e : c->ev_many) cudaEventDestroy(e);
     for (void *p : c->dev_allocs) cudaFree(p);
@@ -1070,8 +1074,8 @@ int hg_step(hg_ctx *c, int64_t n_steps)
     if (n_steps < 0) return fail(c, HG_EINVAL, "n_steps must be >= 0");
     if (n_steps == 0) return HG_OK;
     int rc = sync_bound(c);
+    if (rc == HG_OK) rc = ensure_tnext(c);   // chooses the entry the graphs start from
     if (rc == HG_OK) rc = ensure_graphs(c);
-    if (rc == HG_OK) rc = ensure_tnext(c);
     if (rc) return rc;
     invalidate(c);
     const int64_t s = c->opts.graph_steps;
@@ -1088,8 +1092,8 @@ int hg_advance(hg_ctx *c, double t_end, int64_t *steps_out)
     if (!c) return HG_EINVAL;
     if (!isfinite(t_end)) return fail(c, HG_EINVAL, "t_end must be finite");
     int rc = sync_bound(c);
+    if (rc == HG_OK) rc = ensure_tnext(c);   // chooses the entry the graphs start from
     if (rc == HG_OK) rc = ensure_graphs(c);
-    if (rc == HG_OK) rc = ensure_tnext(c);
     if (rc) return rc;
     invalidate(c);
     rc = sync_scalars(c);

@@ -57,7 +57,10 @@ __global__ void __launch_bounds__(kNBThreads) k_nb_min(const double *tend, int64
     v = LLONG_MAX;
     for (int c = threadIdx.x; c < g; c += blockDim.x) v = min(v, *((volatile long long *)part + c));
     v = block_min_ll(v, sh);
-    if (threadIdx.x == 0) sc->tnext_bits[0] = v;
+    if (threadIdx.x == 0) {
+        sc->tnext_bits[0] = v;
+        sc->slot[0] = 0ull;   // graph steps from here start with an empty list
+    }
 }
 
 __global__ void __launch_bounds__(kNBThreads) k_nb_count(const double *tend, int64_t n, int64_t chunk,
@@ -304,13 +307,6 @@ __global__ void __launch_bounds__(kSelThreads) k_predict_select(const State st, 
     if (!take) return;
     predict_select_pass<MIXED>(st, rec, n, npad, idx, sc, &sc->slot[par], tn, blockIdx.x * (int64_t)blockDim.x + threadIdx.x,
                                (int64_t)gridDim.x * blockDim.x);
-}
-
-// After an odd number of graph steps: entry 0 of the selection's scalars again.
-__global__ void k_swap_entries(DevScalars *sc)
-{
-    sc->tnext_bits[0] = sc->tnext_bits[1];
-    sc->slot[0] = 0ull;
 }
 
 // Predicted FP64 positions and velocities (energy diagnostics).
@@ -1016,12 +1012,6 @@ cudaError_t launch_predict_select(bool mixed, const State &st, const Records &re
     const int g = grid_for(npad, kSelThreads, 1 << 20);
     return launch_dependent(mixed ? k_predict_select<true> : k_predict_select<false>, g, kSelThreads, 0, s, st, rec, n,
                             npad, idx, sc, par);
-}
-
-cudaError_t launch_swap_entries(DevScalars *sc, cudaStream_t s)
-{
-    k_swap_entries<<<1, 1, 0, s>>>(sc);
-    return cudaGetLastError();
 }
 
 cudaError_t launch_predict_clusters(bool mixed, const State &st, const Records &rec, int64_t n, const BatchView &bv,

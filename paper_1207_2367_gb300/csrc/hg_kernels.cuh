@@ -31,7 +31,7 @@ cudaError_t launch_count_due(const State &st, int64_t n, int32_t *cnt, int32_t *
                              const BatchView &bv, cudaStream_t s);
 cudaError_t launch_list_due(const State &st, int64_t n, const int32_t *off, int32_t *idx, DevScalars *sc,
                             cudaStream_t s);
-// Pass 1 alone: sc->tnext_bits[0] = bits of min_i tend_i.
+// Pass 1 alone: sc->tnext_bits[0] = bits of min_i tend_i, sc->slot[0] = 0.
 cudaError_t launch_next_min(const State &st, int64_t n, double *part, DevScalars *sc, cudaStream_t s);
 // One system, graph-replayed block steps: block selection fused into the
 // prediction.  Needs sc->tnext_bits[par] = min_i tend_i and sc->slot[par] = 0 (kept
@@ -39,8 +39,6 @@ cudaError_t launch_next_min(const State &st, int64_t n, double *part, DevScalars
 // particles in idx (arbitrary order), sc->slot[par] of them.
 cudaError_t launch_predict_select(bool mixed, const State &st, const Records &rec, int64_t n, int64_t npad,
                                   int32_t *idx, DevScalars *sc, int par, cudaStream_t s);
-// After an odd number of graph steps: the next one starts from entry 0 again.
-cudaError_t launch_swap_entries(DevScalars *sc, cudaStream_t s);
 // After the state was replaced: tend = t + dt and the FP32 copies (st.f32).
 cudaError_t launch_tend(const State &st, int64_t n, cudaStream_t s);
 // The FP32 copies alone (a no-op for FP64 contexts, st.f32 == nullptr).
