@@ -97,7 +97,8 @@ typedef struct hg_stats {
 
 /* Device time of the block-step sections (Table 1: next-block selection,
  * prediction, evaluation, j-split reduction, correction), accumulated over the
- * graph-replayed block steps taken with opts.profile = 1. */
+ * graph-replayed block steps taken with opts.profile = 1.  The reduction runs inside
+ * the correction's kernel, and the selection of one system inside the prediction's. */
 typedef struct hg_profile {
     double ms[5];          /* next, predict, evaluate, reduce, correct */
     int64_t block_steps;   /* block steps (including no-op steps past t_end) timed */
