@@ -365,7 +365,7 @@ struct Mixed {
 // FP64 path: FP64 records and sums, the pair law in block fixed point on the
 // integer pipes (hg_pair64.cuh).
 // With the whole pair law in FP64 instructions the kernel kept the FP64 unit 91 %
-// busy; m = N = 32768 took 99.4 ms, now 35.6 ms, ~1340 cycles per warp and pair of
+// busy; m = N = 32768 took 99.5 ms, now 36.1 ms, ~1340 cycles per warp and pair of
 // ~690 instructions: a multiply-add with a 64-bit result and a shift or 3-input
 // logic instruction each hold the issue for two cycles.  The nine differences hold
 // the FP64 unit 45 % of the time.  Four blocks per SM (128 registers) measured 1.7 %

@@ -26,8 +26,8 @@
 //   A = q r, J = q w, S = q u with q = m / R^3.
 // Sums: three running exponents per i-particle (A, J, S), raised when a larger
 // term arrives, so that q is shifted once per sum (rounded to nearest) and the
-// products accumulate in 64-bit integers; every kFold64 pairs they are added to
-// FP64 sums.  Errors per pair are 2^-55 or less of |A|, |J|, |S|, against a few
+// products accumulate in 96-bit integers; every kFold64 pairs they are added to
+// FP64 sums (small blocks: the lanes' integers are added first, hg_eval.cu).  Errors per pair are 2^-55 or less of |A|, |J|, |S|, against a few
 // 2^-53 of the FP64 instructions.
 #pragma once
 
