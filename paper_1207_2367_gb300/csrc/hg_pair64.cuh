@@ -218,6 +218,10 @@ HG_P64 int64_t rsqrt_q(uint64_t rho)
 template <bool GUARD>
 HG_P64 bool inverse_radius(int64_t rr, int er2, const Soft &s, int64_t &y, int &hx)
 {
+    // The largest component is 2^(kSVec - 1) or more, and so is its share of rr; the
+    // dropped l l' of the others must not take rr below that: R >= |r| holds with hx.
+    constexpr int64_t kLeast = (int64_t)1 << (2 * (kSVec - 1) - 64);
+    rr = rr > 0 && rr < kLeast ? kLeast : rr;
     int e2 = imax(er2, s.e);
     uint64_t r2 = shr((uint64_t)rr, e2 - er2) + shr((uint64_t)s.q, e2 - s.e);   // < 4
     bool ok = true;
