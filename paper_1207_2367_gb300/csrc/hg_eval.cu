@@ -362,20 +362,17 @@ struct Mixed {
 };
 
 // ------------------------------------------------------------------------
-// FP64 path: FP64 records and sums, the pair law in block fixed point on the
-// integer pipes (hg_pair64.cuh).
+// FP64 path: FP64 records and sums, most of the pair law on the integer pipes
+// (hg_pair64.cuh).
 // With the whole pair law in FP64 instructions the kernel kept the FP64 unit 91 %
-// busy; m = N = 32768 took 99.5 ms, now 36.1 ms, ~1340 cycles per warp and pair of
-// ~690 instructions: a multiply-add with a 64-bit result and a shift or 3-input
-// logic instruction each hold the issue for two cycles.  The nine differences hold
-// the FP64 unit 45 % of the time.  Four blocks per SM (128 registers) measured 1.7 %
-// slower, limbs of 29 bits (every carry and split a shift) 5 %.  Errors against
-// 64-bit arithmetic are below those of the FP64 instructions.
+// busy; m = N = 32768 took 99.5 ms, now 45.6 ms: ~1600 cycles per warp and pair, the FP64
+// unit 83 % busy with 21 instructions, ~850 instructions in all.  Three blocks per SM
+// (168 registers) instead of four (128, small spills): 47.4 ms; two: 52 ms.
 // ------------------------------------------------------------------------
 struct F64 {
     static constexpr int TJ = kTJF64;
     static constexpr int I = 1;
-    static constexpr int kMinBlocks = 2;
+    static constexpr int kMinBlocks = 4;
     static constexpr int kVariant = 0;
     static constexpr uint32_t kStageBytes = TJ * 80;
     struct ITile {
@@ -423,99 +420,68 @@ struct F64 {
         }
     }
 
-    // Sums of up to kFold64 - 1 pairs a lane and 16 lanes or more an i-particle (small
-    // blocks): the lanes' integer sums are added as integers, and lane c converts
-    // component c.  The FP64 instructions of the general path (36 to fold and 45 in the
-    // tree, 64 cycles each) made a block of one particle of 32768 take 20 us, 15 now.
-    __device__ static void epilogue_small(Acc &a, int pairs, int tpi, int tid, double *red, double (&out)[I][kOut])
+    // The N values of this lane and of lane ^ off: the lane whose off bit is clear keeps the
+    // sums of the first (N + 1) / 2, the other one those of the rest.
+    template <int N>
+    __device__ __forceinline__ static void halve(double (&v)[10], int lane, int off)
     {
-        constexpr uint32_t kAll = 0xffffffffu;
-        const int warp = tid >> 5, lane = tid & 31, span = tpi < 32 ? tpi : 32, c = lane & (span - 1);
-        int E[3] = {a.E[0], a.E[1], a.E[2]};
-        uint32_t low = a.low;
-        for (int off = 1; off < span; off <<= 1) {
+        constexpr int H = (N + 1) / 2;
+        const bool up = (lane & off) != 0;
 #pragma unroll
-            for (int g = 0; g < 3; ++g) {
-                const int e = __shfl_xor_sync(kAll, E[g], off);
-                E[g] = e > E[g] ? e : E[g];
-            }
-            const uint32_t l = __shfl_xor_sync(kAll, low, off);
-            low = l < low ? l : low;
+        for (int k = 0; k < H; ++k) {
+            const double hi = H + k < N ? v[H + k] : 0.0;
+            const double give = up ? v[k] : hi, keep = up ? hi : v[k];
+            v[k] = keep + __shfl_xor_sync(0xffffffffu, give, off);
         }
-        p64::align_sums(a, E, pairs * span);
-        for (int off = 1; off < span; off <<= 1) {
-#pragma unroll
-            for (int k = 0; k < 9; ++k) {
-                const int64_t H2 = __shfl_xor_sync(kAll, (long long)a.H[k], off);
-                const uint32_t M2 = __shfl_xor_sync(kAll, a.M[k], off);
-                p64::add_sums(a.H[k], a.M[k], H2, M2);
-            }
-        }
-        int64_t H = a.H[0];
-        uint32_t M = a.M[0];
-#pragma unroll
-        for (int k = 1; k < 9; ++k) {
-            H = c == k ? a.H[k] : H;
-            M = c == k ? a.M[k] : M;
-        }
-        const int e = c < 3 ? a.E[0] : (c < 6 ? a.E[1] : a.E[2]);
-        double v = p64::sum_of(H, M, e, c < 9 ? c : 8);
-        if (low < 0x100000u) v = NAN;
-        if (tpi > 32) {   // two warps an i-particle
-            if (lane < 9) red[warp * kOut + lane] = v;
-            __syncthreads();
-            if (lane < 9) v = red[(warp & ~1) * kOut + lane] + red[(warp | 1) * kOut + lane];
-            __syncthreads();
-        }
-#pragma unroll
-        for (int k = 0; k < 9; ++k) out[0][k] = __shfl_sync(kAll, v, (lane & ~(span - 1)) + k);
-        out[0][9] = 0.0;
     }
 
     // Sum the tpi lanes sharing an i-particle (fixed xor tree; shared memory
     // across warps for tpi = 64): the leader lanes (lane_j == 0) hold out.  No
     // noise scale (out[k][9] = 0): the FP64 path needs no noise floor.
+    // From 16 lanes (small blocks) each level halves the values a lane holds, 9 -> 5 ->
+    // 3 -> 2 -> 1: 11 or 12 additions of 64 cycles instead of 36 or 45 (a block of one
+    // particle of 32768: 14.5 us, 16.7 with them).
     __device__ static void epilogue(Acc &a, int pairs, int tpi, int tid, double *red, double (&out)[I][kOut])
     {
-        if (tpi >= 16 && pairs < p64::kFold64) {   // the same in every thread of the CTA
-            epilogue_small(a, pairs, tpi, tid, red, out);
-            return;
-        }
-        p64::finish(a);
+        constexpr uint32_t kAll = 0xffffffffu;
+        const int warp = tid >> 5, lane = tid & 31;
+        // pairs, of each lane, is the same in every thread of the CTA
+        if (pairs >= p64::kFold64) p64::finish(a);
+        double (&v)[kOut] = out[0];
 #pragma unroll
-        for (int k = 0; k < I; ++k) {
+        for (int c = 0; c < 9; ++c) v[c] = pairs >= p64::kFold64 ? a.s[c] : a.c[c];
+        if (tpi >= 16) {
+            halve<9>(v, lane, 8);
+            halve<5>(v, lane, 4);
+            halve<3>(v, lane, 2);
+            halve<2>(v, lane, 1);
+            double s = v[0];
+            if (tpi >= 32) s += __shfl_xor_sync(kAll, s, 16);
+            // component c is where the bits 8, 4, 2, 1 of the lane took it
 #pragma unroll
-            for (int c = 0; c < 9; ++c) out[k][c] = a.s[c];
-            out[k][9] = 0.0;
-        }
-        const int wspan = tpi < 32 ? tpi : 32;
-        for (int off = 1; off < wspan; off <<= 1) {
-#pragma unroll
-            for (int k = 0; k < I; ++k)
-#pragma unroll
-                for (int c = 0; c < 9; ++c) out[k][c] += __shfl_xor_sync(0xffffffffu, out[k][c], off);
-        }
-        if (tpi > 32) {
-            const int warp = tid >> 5, lane = tid & 31, wpg = tpi >> 5;
-            if (lane == 0) {
-#pragma unroll
-                for (int k = 0; k < I; ++k)
-#pragma unroll
-                    for (int c = 0; c < 9; ++c) red[(warp * I + k) * kOut + c] = out[k][c];
+            for (int c = 0; c < 9; ++c) {
+                const int c1 = c < 5 ? c : c - 5, c2 = c1 < 3 ? c1 : c1 - 3, c3 = c2 < 2 ? c2 : c2 - 2;
+                const int src = (c < 5 ? 0 : 8) + (c1 < 3 ? 0 : 4) + (c2 < 2 ? 0 : 2) + c3;
+                v[c] = __shfl_sync(kAll, s, (lane & 16) + src);
             }
-            __syncthreads();
-            if (lane == 0 && (warp % wpg) == 0) {
+            if (tpi > 32) {   // two warps an i-particle
+                double w = 0.0;
 #pragma unroll
-                for (int k = 0; k < I; ++k)
+                for (int c = 0; c < 9; ++c) w = lane == c ? v[c] : w;
+                if (lane < 9) red[warp * kOut + lane] = w;
+                __syncthreads();
+                if (lane < 9) w = red[(warp & ~1) * kOut + lane] + red[(warp | 1) * kOut + lane];
 #pragma unroll
-                    for (int c = 0; c < 9; ++c) {
-                        double s = red[(warp * I + k) * kOut + c];
-                        for (int g = 1; g < wpg; ++g) s += red[((warp + g) * I + k) * kOut + c];
-                        out[k][c] = s;
-                    }
+                for (int c = 0; c < 9; ++c) v[c] = __shfl_sync(kAll, w, c);
+                __syncthreads();
             }
-            __syncthreads();
+        } else {
+            for (int off = 1; off < tpi; off <<= 1) {
+#pragma unroll
+                for (int c = 0; c < 9; ++c) v[c] += __shfl_xor_sync(kAll, v[c], off);
+            }
         }
+        v[9] = 0.0;
     }
 };
 

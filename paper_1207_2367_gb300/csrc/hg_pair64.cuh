@@ -1,38 +1,38 @@
-// hg_pair64.cuh -- the FP64 path's pair law on the integer pipes: acceleration,
-// jerk and snap of a pair, and a pair's potential, at FP64 accuracy or better
-// without the FP64 unit (host and device; the host form serves the CPU test).
+// hg_pair64.cuh -- the FP64 path's pair law (acceleration, jerk and snap of a pair) and a
+// pair's potential (host and device; the host form serves the CPU tests).
 //
 // GB300 has two FP64 lanes per SM: a warp-wide FP64 instruction holds its
-// sub-partition's unit for 64 cycles, so the ~55 FP64 instructions of a pair are
-// ~3500 cycles per warp.  A 32 x 32 + 64-bit integer multiply-add takes two.  Here
-// only the differences r_j - r_i, v_j - v_i, a_j - a_i (nine subtractions, whose
-// operands have any exponents) are FP64 instructions; everything after them is
-// block fixed point.
+// sub-partition's unit for 64 cycles, so a pair law of ~55 FP64 instructions takes
+// ~3500 cycles per warp.  A 32 x 32 + 64-bit integer multiply-add takes two.  Hence only
+//   the differences r, v, a, w = v - 3 alpha r and the sums of q r, q w and q u
+// are FP64 instructions (21), and the rest runs on the integer pipes beside them:
+//   R^2 = r^2 + eps^2, q = m / R^3, alpha = r.v / R^2,
+//   u = a - 6 alpha v - gamma r, gamma = 3 (v^2 + r.a) / R^2 - 15 alpha^2.
 //
-// Numbers are 64-bit integers: x stands for X = x 2^S with a scale S known at each
-// place, beside a binary exponent; each of the vectors r, v, a has one exponent (its
-// largest component lies in [1/2, 1)), so a component is exact to 2^-62 of the
-// vector's size.  A factor of a product is split at its 32nd bit, X = h 2^32 + l with
-// l signed (its word as it is; h takes the carry), and X Y / 2^64 = h h' +
-// (h l' + l h') / 2^32: the word of a sum is its quotient, so a product is four
-// multiply-adds (l l' is below its last place) and no shift, dot products and sums
-// accumulating inside them.  The scales below are chosen so that |h| < 2^31 and
-// that the cross sums stay below 2^63 (the |h| of the factors add up to < 2^32).
+// Integer numbers are 64-bit sizes with a sign and a binary exponent of their own: every
+// product of a dot product and every component of u has its exponent, and the terms of
+// a sum are shifted to the largest of them.  So a component of the sums is as good
+// whatever the others are (thin discs, nearly aligned pairs).  The integers lose 2^-55 or
+// so of the sizes of a component's terms and are rounded to FP64 once: a pair's terms are
+// within 3 2^-53 of these sizes, where FP64 instructions throughout reach 8 (q r), 15
+// (q w) and 16 (q u) 2^-53 (10^6 random pairs each, of seven kinds).  A factor of a product is
+// split at its 32nd bit, X = h 2^32 + l, and X Y / 2^64 = h h' + (h l' + l h') / 2^32:
+// three multiply-adds (l l' is below the last place).  Infinities, NaN and
+// numbers near the ends of FP64's range are left to FP64 instructions (vectors_fp64); a
+// component of u all of whose terms are below 2^-762 may count as zero.
 //
-// The pair law, with R^2 = r^2 + eps^2 and n = r / R (so that every factor is
-// bounded by the vectors it multiplies):
-//   lambda = n.v, nu = n.a, w = v - 3 lambda n,
-//   u = a - 3 nu n - (6 lambda w + 3 (v^2 + lambda^2) n) / R,
-//   A = q r, J = q w, S = q u with q = m / R^3.
-// Sums: three running exponents per i-particle (A, J, S), raised when a larger
-// term arrives, so that q is shifted once per sum (rounded to nearest) and the
-// products accumulate in 96-bit integers; every kFold64 pairs they are added to
-// FP64 sums (small blocks: the lanes' integers are added first, hg_eval.cu).  Errors per pair are 2^-55 or less of |A|, |J|, |S|, against a few
-// 2^-53 of the FP64 instructions.
+// An evaluation of N = 32768 particles: 45.6 ms, the FP64 unit 83 % busy; with w in integers
+// too (18 FP64 instructions) 49.1 ms; with u in FP64 instructions as well the unit alone would
+// take 48 ms.  (One exponent for the three components of a vector and of a sum takes 36 ms,
+// but holds small components in fewer bits than FP64 does.)
+//
+// The potential of a pair is one positive number, m / R: integers after the three
+// differences, sums over kFold64 pairs in block fixed point.
 #pragma once
 
 #include <math.h>
 #include <stdint.h>
+#include <string.h>
 
 #include "hg_internal.cuh"
 
@@ -45,19 +45,13 @@ namespace p64 {
 #define HG_P64 inline
 #endif
 
-constexpr int kSVec = 62;                 // scale of r, v, a
-constexpr int kSMass = 63;                // of the mass, in [1/4, 1/2)
+constexpr int kSVec = 62;                 // scale of the potential's separation
+constexpr int kSMass = 63;                // of its mass, in [1/4, 1/2)
 constexpr int kSR2 = 2 * kSVec - 64;      // of r^2 and eps^2
 constexpr int kSY = 61;                   // of y, in (1, 2]
-constexpr int kSQ = 61;                   // of q, in [1/4, 4)
-constexpr int kFold64 = 32;               // pairs between additions to the FP64 sums
-// A term enters its sum with |q'| < 2^kBitsQ: the high sums of kFold64 terms stay
-// below 32 * 2^(59 - 32) * 3.5 * 2^29 < 2^63; a dropped l l' is 2^-56 of the largest
-// term.  A sum's exponent is raised by kSlack more than a larger term needs, so that
-// it moves less often.
-constexpr int kBitsQ = 59, kSlack = 2;
-constexpr int kExpNone = -(1 << 28);      // exponent of an empty sum
-static_assert(kFold64 == 32, "the room of align_sums");
+constexpr int kFold64 = 32;               // pairs between additions to the total sums
+constexpr int kSlack = 2;                 // its exponent is raised by this much more than needed
+constexpr int kExpNone = -(1 << 28);      // exponent of zero
 
 struct Limbs {
     int32_t h, l;
@@ -132,13 +126,6 @@ HG_P64 int64_t carry(int64_t H, int64_t M) { return mad(hi32(M), 1, H); }
 // sign, since the sums run over many pairs whose terms cancel.
 constexpr int64_t kRound = (int64_t)1 << 31;
 HG_P64 int64_t mul(Limbs a, Limbs b) { return carry(mad(a.h, b.h, 0), mad(a.h, b.l, mad(a.l, b.h, kRound))); }
-HG_P64 int64_t sqr(Limbs a) { return mad(hi32(mad(a.h, a.l, kRound >> 1)), 2, mad(a.h, a.h, 0)); }
-HG_P64 int64_t dot(const Limbs (&a)[3], const Limbs (&b)[3])
-{
-    return carry(mad(a[2].h, b[2].h, mad(a[1].h, b[1].h, mad(a[0].h, b[0].h, 0))),
-                 mad(a[2].h, b[2].l, mad(a[2].l, b[2].h, mad(a[1].h, b[1].l, mad(a[1].l, b[1].h,
-                     mad(a[0].h, b[0].l, mad(a[0].l, b[0].h, kRound)))))));
-}
 HG_P64 int64_t norm2(const Limbs (&a)[3])
 {
     return mad(hi32(mad(a[2].h, a[2].l, mad(a[1].h, a[1].l, mad(a[0].h, a[0].l, kRound >> 1)))), 2,
@@ -168,10 +155,12 @@ HG_P64 int vec(double d0, double d1, double d2, int64_t (&o)[3], uint32_t &low)
     return 2047 - ne - 1022;
 }
 
-// eps^2 as a fraction in [1/2, 1) (scale kSR2) and its exponent; zero: fraction 0, no exponent.
+// eps^2 as a fraction in [1/2, 1) (scale kSR2) and its exponent; zero: fraction 0, no exponent;
+// beyond FP64's range: an exponent that leaves q below it.
 struct Soft {
     int64_t q;
     int e;
+    double eps2;
 };
 inline
 #if defined(__CUDACC__)
@@ -179,12 +168,13 @@ inline
 #endif
     Soft soft(double eps2)
 {
-    Soft s{0, kExpNone};
+    Soft s{0, kExpNone, eps2};
     if (eps2 > 0.0) {
         int e;
-        const double f = frexp(eps2, &e);   // [1/2, 1)
+        const bool finite = eps2 < INFINITY;
+        const double f = frexp(finite ? eps2 : 1.0, &e);   // [1/2, 1)
         s.q = (int64_t)ldexp(f, kSR2);
-        s.e = e;
+        s.e = finite ? e : 8192;
     }
     return s;
 }
@@ -214,16 +204,13 @@ HG_P64 int64_t rsqrt_q(uint64_t rho)
 }
 
 // R^2 = r^2 + eps^2 = (rho / 2^64) 2^(2 hx) and y = (rho / 2^64)^(-1/2), from
-// r^2 = rr 2^er2.  Returns false (y = 1, hx = 0) for R^2 = 0 or below FP64's range.
+// r^2 = rr 2^(er2 - kSR2), rr < 2^63.  Returns false (y = 1, hx = 0) for R^2 = 0 or below
+// FP64's range.
 template <bool GUARD>
 HG_P64 bool inverse_radius(int64_t rr, int er2, const Soft &s, int64_t &y, int &hx)
 {
-    // The largest component is 2^(kSVec - 1) or more, and so is its share of rr; the
-    // dropped l l' of the others must not take rr below that: R >= |r| holds with hx.
-    constexpr int64_t kLeast = (int64_t)1 << (2 * (kSVec - 1) - 64);
-    rr = rr > 0 && rr < kLeast ? kLeast : rr;
     int e2 = imax(er2, s.e);
-    uint64_t r2 = shr((uint64_t)rr, e2 - er2) + shr((uint64_t)s.q, e2 - s.e);   // < 4
+    uint64_t r2 = shr((uint64_t)rr, e2 - er2) + shr((uint64_t)s.q, e2 - s.e);
     bool ok = true;
     if (GUARD) {
         ok = r2 != 0 && e2 > -1074;
@@ -250,69 +237,225 @@ HG_P64 int mass_limbs(double m, Limbs &o, uint32_t &low)
     return imax(e, 1) - 1021;
 }
 
+// Size of a normal double or zero: x 2^(e - 1085), the top bit of x at bit 62; zero is 0 with
+// e = kExpZero, below any product's exponent.  A denormal number (x > 0 with kExpZero)
+// counts for nothing beside the others; vectors_int bounds what it could have been.
+constexpr int kExpZero = -8192;
+struct Size {
+    uint64_t x;
+    int e;
+};
+HG_P64 Size size_of(double d)
+{
+    const uint64_t b = dbits(d);
+    const uint32_t lo = (uint32_t)b, ah = (uint32_t)(b >> 32) & 0x7fffffffu;
+    const uint32_t top = (ah & 0xfffffu) | umin(ah, 0x100000u);
+    return Size{(uint64_t)word((int32_t)((top << 10) | (lo >> 22)), (int32_t)(lo << 10)),
+                ah >= 0x100000u ? (int)(ah >> 20) : kExpZero};
+}
+HG_P64 int max_e(const Size (&s)[3]) { return imax(imax(s[0].e, s[1].e), s[2].e); }
+
+// All bits of a sign: 0 or -1.
+HG_P64 int32_t sign_of(double d) { return hi32((int64_t)dbits(d)) >> 31; }
+HG_P64 int32_t sign_of(int64_t x) { return hi32(x) >> 31; }
+// X + x or, for s = -1, X - x.
+HG_P64 int64_t add_signed(int64_t X, uint64_t x, int32_t s) { return X + (int64_t)(x ^ (uint64_t)word(s, s)) - s; }
+
+// x y / 2^64 and x^2 / 2^64 to within a unit, for x, y <= 2^63.
+HG_P64 uint64_t mulu(uint64_t x, uint64_t y)
+{
+    const uint32_t h = (uint32_t)(x >> 32), l = (uint32_t)x, h2 = (uint32_t)(y >> 32), l2 = (uint32_t)y;
+    return madu(h, h2, madu(h, l2, madu(l, h2, 0x80000000u)) >> 32);
+}
+HG_P64 uint64_t squ(uint64_t x)
+{
+    const uint32_t h = (uint32_t)(x >> 32), l = (uint32_t)x;
+    return madu(h, h, madu(h, l, 0x40000000u) >> 31);
+}
+
+HG_P64 int clz64(uint64_t x)
+{
+#if defined(__CUDA_ARCH__)
+    return __clzll((long long)x);
+#else
+    return x ? __builtin_clzll(x) : 64;
+#endif
+}
+
+// Number x 2^e (x > 0: top bit at bit 62; zero: any e, kExpNone from normal) with the sign s.
+struct Number {
+    uint64_t x;
+    int e;
+    int32_t s;
+};
+// X 2^e for |X| < 2^63, turned over for s = -1.
+HG_P64 Number normal(int64_t X, int e, int32_t s)
+{
+    Number n;
+    const int32_t sx = sign_of(X);
+    const uint64_t x = (uint64_t)add_signed(0, (uint64_t)X, sx);
+    const int z = clz64(x) - 1;
+    n.x = x << z;
+    n.e = z < 63 ? e - z : kExpNone;
+    n.s = s ^ sx;
+    return n;
+}
+
+// x 2^e for x = 0 or x in [2^32, 2^63).
+HG_P64 Number normal_hi(uint64_t x, int e, int32_t s)
+{
+    const int z = clz32((uint32_t)(x >> 32)) - 1;
+    return Number{x << z, e - z, s};
+}
+
+// Rounded to FP64; ok turns false for what is not zero and not a normal number.
+HG_P64 double to_fp64(const Number &n, bool &ok)
+{
+    const int eb = n.e + (62 + 1022);                     // exponent field less one, before rounding
+    ok = ok && ((uint32_t)eb < 2045u || hi32((int64_t)n.x) == 0);
+    const uint64_t m = (n.x + 0x200u) >> 10;              // the top bit, in place 52, adds one to the field
+    const uint64_t b = m + ((uint64_t)((uint32_t)imax(eb, 0) << 20 | ((uint32_t)n.s & 0x80000000u)) << 32);
+#if defined(__CUDA_ARCH__)
+    return __longlong_as_double((long long)b);
+#else
+    double d;
+    memcpy(&d, &b, 8);
+    return d;
+#endif
+}
+
+// What a pair adds to the sums: q r, q w, q u.
+struct Terms {
+    double q, w[3], u[3];
+};
+
+// In FP64 instructions: any inputs.
+template <bool GUARD>
+HG_P64 void vectors_fp64(const double (&r)[3], const double (&v)[3], const double (&a)[3], double m, double eps2,
+                         Terms &t)
+{
+    const double r2 = fma(r[2], r[2], fma(r[1], r[1], fma(r[0], r[0], eps2)));
+#if defined(__CUDA_ARCH__)
+    double rinv = rsqrt(r2);
+#else
+    double rinv = 1.0 / sqrt(r2);
+#endif
+    if (GUARD) rinv = (r2 > 0.0) ? rinv : 0.0;
+    const double rinv2 = rinv * rinv;
+    const double rv = fma(r[2], v[2], fma(r[1], v[1], r[0] * v[0]));
+    const double v2ra = fma(r[2], a[2], fma(r[1], a[1], fma(r[0], a[0], fma(v[2], v[2], fma(v[1], v[1], v[0] * v[0])))));
+    const double alpha = rv * rinv2;
+    const double a3 = -3.0 * alpha, b3 = -3.0 * fma(alpha, alpha, v2ra * rinv2);
+    t.q = m * rinv * rinv2;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        t.w[k] = fma(a3, r[k], v[k]);
+        t.u[k] = fma(b3, r[k], fma(a3 + a3, t.w[k], a[k]));
+    }
+}
+
+// In integers but for w; returns false for what they do not hold.
+template <bool GUARD>
+HG_P64 bool vectors_int(const double (&r)[3], const double (&v)[3], const double (&a)[3], double m, const Soft &soft2,
+                        Terms &t)
+{
+    const Size rs[3] = {size_of(r[0]), size_of(r[1]), size_of(r[2])};
+    const Size vs[3] = {size_of(v[0]), size_of(v[1]), size_of(v[2])};
+    const Size as[3] = {size_of(a[0]), size_of(a[1]), size_of(a[2])};
+    const Size ms = size_of(m);
+    const int32_t sr[3] = {sign_of(r[0]), sign_of(r[1]), sign_of(r[2])};
+    const int32_t sv[3] = {sign_of(v[0]), sign_of(v[1]), sign_of(v[2])};
+    const int32_t sa[3] = {sign_of(a[0]), sign_of(a[1]), sign_of(a[2])};
+    const int er = max_e(rs), ev = max_e(vs);
+    // Here and below, ok holds the numbers to a range in which denormal components (below
+    // 2^-1022) have no part of 2^-62 in any sum: components below 2^500, dot products with a
+    // term of 2^-460 or more, alpha and gamma below 2^260, u with a term of 2^-700 or more
+    // (or all terms zero).
+    bool ok = imax(imax(er, ev), max_e(as)) < 1023 + 500 && ms.e < 2047;
+
+    // r^2 = rr 2^(2 er - 2105): products below 2^62 (2^60 or more for the largest), halved.
+    uint64_t rr = 0;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) rr += shr(squ(rs[k].x), 2 * (er - rs[k].e) + 1);
+    int64_t yi;
+    int hx;
+    const bool apart = inverse_radius<GUARD>((int64_t)rr, 2 * er - 2045, soft2, yi, hx);
+    const uint64_t y = (uint64_t)yi << 1;                  // 1/R = y 2^(-62 - hx), y in (2^62, 2^63]
+    const uint64_t y2 = squ(y), y3 = (3 * y2) >> 1;        // 1/R^2 = y2 2^(-60 - 2 hx), 3/R^2 = y3 2^(-59 - 2 hx)
+
+    // r.v, below 3 2^61 in units of 2^(e1 - 2105); v^2 + r.a, below 6 2^60 in units of 2^(e2 - 2104)
+    int p[3], c[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        p[k] = rs[k].e + vs[k].e;
+        c[k] = rs[k].e + as[k].e;
+    }
+    const int e1 = imax(imax(p[0], p[1]), p[2]), e2 = imax(imax(imax(c[0], c[1]), c[2]), 2 * ev);
+    ok = ok && (uint32_t)e1 >= 2046u - 460u && (uint32_t)e2 >= 2046u - 460u;   // (or negative)
+    const int32_t s0 = sr[0] ^ sv[0];
+    int64_t X = (int64_t)shr(mulu(rs[0].x, vs[0].x), e1 - p[0] + 1), Z = 0;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        if (k > 0) X = add_signed(X, shr(mulu(rs[k].x, vs[k].x), e1 - p[k] + 1), sr[k] ^ sv[k] ^ s0);
+        Z += (int64_t)shr(squ(vs[k].x), e2 - 2 * vs[k].e + 2);
+        Z = add_signed(Z, shr(mulu(rs[k].x, as[k].x), e2 - c[k] + 2), sr[k] ^ sa[k]);
+    }
+    const Number rv = normal(X, e1 - 2105, s0), va = normal(Z, e2 - 2104, 0);
+
+    // 3 alpha = al3 2^ea, al3 < 3 2^60; alpha = al 2^(ea - 1), al <= 2^61
+    const uint64_t al3 = mulu(rv.x, y3), al = mulu(rv.x, y2);
+    const int ea = rv.e + 64 - 59 - 2 * hx;
+    // gamma = ga 2^eg: its parts below 3 2^60 and 15 2^57
+    const int eg1 = va.e + 64 - 59 - 2 * hx, eg2 = 2 * ea + 63, eg = imax(eg1, eg2);
+    const int64_t G = add_signed(-(int64_t)shr(mulu((al << 1) + (al >> 1), al3 << 1), eg - eg2),
+                                 shr(mulu(va.x, y3), eg - eg1), va.s);
+    ok = ok && imax(ea, eg) < 260 - 62;
+    const int32_t sg = sign_of(G);
+    const uint64_t ga = (uint64_t)add_signed(0, (uint64_t)G, sg);
+
+    const double a3 = to_fp64(normal_hi(al3, ea, ~rv.s), ok);
+
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        t.w[k] = fma(a3, r[k], v[k]);
+        // u: a_k below 2^61, 6 alpha v_k below 3 2^59, gamma r_k below 2^62, in units of 2^(eu + 2)
+        const int fa = as[k].e - 1085, fw = ea + vs[k].e + (65 - 1085), fg = eg + rs[k].e + (64 - 1085);
+        const int eu = imax(imax(fa, fw - 2), fg - 2);
+        ok = ok && (uint32_t)(eu + 4096) >= 4096u - 700u;   // (or below -4096)
+        const Number u = normal(add_signed(add_signed((int64_t)shr(as[k].x, eu - fa + 2),
+                                                      shr(mulu(al3, vs[k].x), eu - fw + 2), ~(rv.s ^ sv[k] ^ sa[k])),
+                                           shr(mulu(ga, rs[k].x), eu - fg + 2), ~(sg ^ sr[k] ^ sa[k])),
+                                eu + 2, sa[k]);
+        t.u[k] = to_fp64(u, ok);
+    }
+    // m / R^3 = m (1/R) (1/R^2), below 2^62
+    t.q = to_fp64(normal((int64_t)mulu(mulu(ms.x, y), y2 << 1), ms.e - 1080 - 3 * hx, sign_of(m)), ok);
+    if (GUARD && !apart) t.q = 0.0;   // a pair at zero distance
+    return ok;
+}
+
 // i-particle: position, velocity, acceleration.
 struct Body {
     double x, y, z, vx, vy, vz, ax, ay, az;
 };
 
-// Sums of one i-particle on one lane.  Component c: (H[c] + M[c] / 2^32) in units of
-// 2^(E[c/3] - unit(c/3)), beside s.
+// Sums of one i-particle on one lane: c over up to kFold64 pairs, s of the finished ones (so
+// that a large term meets few roundings at its own size).
 struct Sums {
-    int64_t H[9];
-    uint32_t M[9];
-    int E[3];
-    double s[9];
-    int cnt;         // pairs since the last addition to s
-    uint32_t low;    // smallest complemented high word of a difference or mass (infinities, NaN)
+    double c[9], s[9];
+    int cnt;         // pairs in c
+#if !defined(__CUDACC__)
+    bool bad;        // host checks: an infinity or NaN among the pairs (shown in every sum)
+#endif
 };
-// Scales of r, w, u where they enter the sums; the sums' units.
-constexpr int kSW = 61, kSU = 61;
-HG_P64 int unit(int g) { return kSQ + (g == 0 ? kSVec : g == 1 ? kSW : kSU) - 64; }
 
 HG_P64 void clear(Sums &a)
 {
-    for (int c = 0; c < 9; ++c) {
-        a.H[c] = 0;
-        a.M[c] = 0u;
-        a.s[c] = 0.0;
-    }
-    for (int g = 0; g < 3; ++g) a.E[g] = kExpNone;
+    for (int k = 0; k < 9; ++k) a.c[k] = a.s[k] = 0.0;
     a.cnt = 0;
-    a.low = 0x7fffffffu;
-}
-
-// q 2^-s rounded to nearest (s >= 1), as limbs.
-HG_P64 Limbs scaled(int64_t q, int s) { return split((sar(q, s - 1) + 1) >> 1); }
-
-HG_P64 void add_term(Sums &a, int g, Limbs q, const Limbs (&x)[3])
-{
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        const int64_t m = mad(q.h, x[k].l, mad(q.l, x[k].h, (int64_t)(uint64_t)a.M[3 * g + k]));
-        a.M[3 * g + k] = (uint32_t)lo32(m);
-        a.H[3 * g + k] = carry(mad(q.h, x[k].h, a.H[3 * g + k]), m);
-    }
-}
-
-// (H, M) 2^-d; from d = 32 on the rest below H's last place is dropped.
-HG_P64 void shift_sum(int64_t &H, uint32_t &M, int d)
-{
-    M = d < 32 ? (uint32_t)lo32((int64_t)shr((uint64_t)word(lo32(H), (int32_t)M), d)) : 0u;
-    H = sar(H, d);
-}
-
-// A term larger than the sums' units allow moves them to its exponent.
-HG_P64 void raise(Sums &a, const int (&need)[3])
-{
-#pragma unroll
-    for (int g = 0; g < 3; ++g) {
-        const int d = need[g] > a.E[g] ? need[g] + kSlack - a.E[g] : 0;
-        a.E[g] += d;
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            shift_sum(a.H[3 * g + k], a.M[3 * g + k], d);
-        }
-    }
+#if !defined(__CUDACC__)
+    a.bad = false;
+#endif
 }
 
 // One pair: j-particle (position, mass, velocity, acceleration) on i-particle d.
@@ -320,70 +463,45 @@ template <bool GUARD>
 HG_P64 void pair(const Body &d, double jx, double jy, double jz, double jm, double jvx, double jvy, double jvz,
                  double jax, double jay, double jaz, const Soft &soft2, Sums &acc)
 {
-    int64_t rx[3], vx[3], ax[3];
-    Limbs r[3], v[3], a[3], m;
-    const int er = vec(jx - d.x, jy - d.y, jz - d.z, rx, acc.low);
-    const int ev = vec(jvx - d.vx, jvy - d.vy, jvz - d.vz, vx, acc.low);
-    const int ea = vec(jax - d.ax, jay - d.ay, jaz - d.az, ax, acc.low);
-    const int em = mass_limbs(jm, m, acc.low);
+    const double r[3] = {jx - d.x, jy - d.y, jz - d.z};
+    const double v[3] = {jvx - d.vx, jvy - d.vy, jvz - d.vz};
+    const double a[3] = {jax - d.ax, jay - d.ay, jaz - d.az};
+    Terms t;
+    if (!vectors_int<GUARD>(r, v, a, jm, soft2, t)) vectors_fp64<GUARD>(r, v, a, jm, soft2.eps2, t);
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        r[k] = split(rx[k]);
-        v[k] = split(vx[k]);
-        a[k] = split(ax[k]);
+        acc.c[k] = fma(t.q, r[k], acc.c[k]);
+        acc.c[3 + k] = fma(t.q, t.w[k], acc.c[3 + k]);
+        acc.c[6 + k] = fma(t.q, t.u[k], acc.c[6 + k]);
     }
+#if !defined(__CUDACC__)
+    for (int k = 0; k < 3; ++k) acc.bad = acc.bad || !isfinite(r[k]) || !isfinite(v[k]) || !isfinite(a[k]);
+    acc.bad = acc.bad || !isfinite(jm);
+#endif
+}
 
-    int64_t y;
-    int hx;
-    const bool ok = inverse_radius<GUARD>(norm2(r), 2 * er, soft2, y, hx);
-    if (GUARD && !ok) return;   // a pair at zero distance
-    const Limbs yl = split(y);
-    // q = m y^3 2^(em - 3 hx), in [1/4, 4): (m y) and y^2 lifted to scales 62 and 60
-    const int64_t q = mul(split(mul(m, yl) << 2), split(sqr(yl) << 2)) << 3;
-
-    // n = r / R = n' 2^-hn: below R = 2 r or so n' stays of order one (|n'| < 1.75).
-    const int s1 = imin(hx - er, 1), hn = hx - er - s1;
-    const Limbs ys = split(y >> s1);
-    Limbs n[3];                                          // scale 59
+HG_P64 void fold(Sums &a)
+{
 #pragma unroll
-    for (int k = 0; k < 3; ++k) n[k] = split(mul(r[k], ys));
-
-    // lambda = lam 2^-hn, nu = nu' 2^-hn, |lam| and |nu'| < 3.1 (< 1.75 for hn = 0), scale 57
-    const int64_t lam = dot(n, v), nu = dot(n, a);
-    const Limbs ll = split(lam << 4);                    // scale 61
-    const Limbs l3 = split(sar(3 * lam, 2 * hn) << 3);   // 3 lambda 2^-hn < 5.3, scale 60
-    Limbs w[3];
-#pragma unroll
-    for (int k = 0; k < 3; ++k)                          // |w| <= 2 |v| < 3.5
-        w[k] = split((vx[k] >> (kSVec - kSW)) - (mul(l3, n[k]) << (kSW - 55)));
-    // kappa = (v^2 + lambda^2) y / 2 <= 6, scale 58.  The part of u along 1 / R has the
-    // length |6 (lambda y w + kappa n)| <= 6 kappa (its square over y^2 v^4 |n|^2, with c
-    // the cosine of v and n, is (3 + 6 c^2 - 15 |n|^2 c^2)^2 + 36 c^2 (1 - c^2)), and at
-    // most 32 kappa |n| / |n'|; |a - 3 nu n| <= 2 |a| < 3.5.
-    const int64_t kap = mul(split(norm2(v) + (sar(sqr(ll), 2 * hn) << 2)), yl);
-    const int64_t lam1 = mul(ll, yl);                    // scale 58
-    const int bk = 6 - imin(clz32((uint32_t)hi32(kap)), 7);   // kappa < 2^bk, bk >= -1
-    const int ec = 2 * ev - hx - hn;
-    const int eu = imax(ea + 2, ec + bk + 2 + imin(hn, 3));
-    const int sa = eu - ea, sz = eu - ec - 1;            // >= 2, >= bk + 1
-    const Limbs c1 = split(sar(12 * nu, sa + 2 * hn - 2) + (sar(3 * kap, sz) << 3) + 4);   // < 2.9, scale 61
-    const Limbs c2 = split(sar(3 * lam1, sz) << 1);                                        // <= 3, scale 59
-    Limbs u[3];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {                        // |u| < 2.4, formed at scale 56, lifted
-        const int64_t H = mad(c2.h, w[k].h, mad(c1.h, n[k].h, 0));
-        const int64_t M = mad(c2.h, w[k].l, mad(c2.l, w[k].h, mad(c1.h, n[k].l, mad(c1.l, n[k].h, kRound))));
-        u[k] = split(sar(ax[k], sa + kSVec - kSU) - (carry(H, M) << (kSU - 56)));
+    for (int k = 0; k < 9; ++k) {
+        a.s[k] += a.c[k];
+        a.c[k] = 0.0;
     }
+    a.cnt = 0;
+}
+HG_P64 void count_pair(Sums &a)
+{
+    if (++a.cnt == kFold64) fold(a);
+}
 
-    // The sums: |q| < 2^b, brought below 2^kBitsQ in each sum's units.
-    const int eq = em - 3 * hx;
-    const int b = 64 - imin(clz32((uint32_t)hi32(q < 0 ? -q : q)), 5) - kBitsQ + eq;
-    const int need[3] = {b + er, b + ev, b + eu};
-    if (imax(imax(need[0] - acc.E[0], need[1] - acc.E[1]), need[2] - acc.E[2]) > 0) raise(acc, need);
-    add_term(acc, 0, scaled(q, acc.E[0] - eq - er), r);
-    add_term(acc, 1, scaled(q, acc.E[1] - eq - ev), w);
-    add_term(acc, 2, scaled(q, acc.E[2] - eq - eu), u);
+// All sums in s.
+HG_P64 void finish(Sums &a)
+{
+    fold(a);
+#if !defined(__CUDACC__)
+    for (double &x : a.s)
+        if (a.bad) x = NAN;
+#endif
 }
 
 // 2^e for |e| <= 1022.
@@ -404,56 +522,6 @@ HG_P64 double add_scaled(double s, int64_t H, int e)
     if (e >= -960 && e <= 960) return fma(h, exp2i(e), s);
     const int c = imin(imax(e, -2040), 2040), c1 = c >> 1;
     return s + (h * exp2i(c1)) * exp2i(c - c1);
-}
-
-// The high sums into the FP64 sums.
-HG_P64 void fold_fp64(Sums &a)
-{
-#pragma unroll
-    for (int c = 0; c < 9; ++c) {
-        a.s[c] = add_scaled(a.s[c], a.H[c], a.E[c / 3] - unit(c / 3));
-        a.H[c] = 0;
-    }
-    a.cnt = 0;
-}
-
-// Component c of the integer sums alone.
-HG_P64 double sum_of(int64_t H, uint32_t M, int E, int c)
-{
-    const int e = E - unit(c / 3);
-    return add_scaled(add_scaled(0.0, H, e), (int64_t)(uint64_t)M, e - 32);
-}
-
-// Sums of lanes that together took `all` pairs, the same number each and none folded
-// yet: moves this lane's to the exponents E, with room for the total.
-HG_P64 void align_sums(Sums &a, const int (&E)[3], int all)
-{
-    const int room = all > kFold64 ? 32 - clz32((uint32_t)(all - 1)) - 5 : 0;
-#pragma unroll
-    for (int c = 0; c < 9; ++c) shift_sum(a.H[c], a.M[c], E[c / 3] + room - a.E[c / 3]);
-    for (int g = 0; g < 3; ++g) a.E[g] = E[g] + room;
-}
-HG_P64 void add_sums(int64_t &H, uint32_t &M, int64_t H2, uint32_t M2)
-{
-    const uint64_t m = (uint64_t)M + M2;
-    M = (uint32_t)m;
-    H += H2 + (int64_t)(m >> 32);
-}
-
-HG_P64 void count_pair(Sums &a)
-{
-    if (++a.cnt == kFold64) fold_fp64(a);
-}
-
-// All sums in s; an infinity or NaN among the inputs gives NaN.
-HG_P64 void finish(Sums &a)
-{
-    fold_fp64(a);
-#pragma unroll
-    for (int c = 0; c < 9; ++c) {
-        a.s[c] = add_scaled(a.s[c], (int64_t)(uint64_t)a.M[c], a.E[c / 3] - unit(c / 3) - 32);
-        if (a.low < 0x100000u) a.s[c] = NAN;
-    }
 }
 
 // Potential of one pair, m / R (R^2 = r^2 + eps^2): H 2^(E - kSPot) sums the pairs
