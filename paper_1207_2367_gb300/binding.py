@@ -200,6 +200,10 @@ def hg_predict(ctx, t):
 
 
 def hg_evaluate(ctx, idx, m, acc=None, jerk=None, snap=None):
+    need = 3 * int(m)
+    for a in (acc, jerk, snap):   # device arrays are written by a kernel
+        if a is not None and (a.size if isinstance(a, np.ndarray) else a.numel()) < need:
+            raise ValueError(f"a result array holds fewer than 3 x {int(m)} values")
     _check(ctx, load().hg_evaluate(ctx, _ptr(idx, np.int32), int(m), _ptr(acc), _ptr(jerk), _ptr(snap)))
 
 

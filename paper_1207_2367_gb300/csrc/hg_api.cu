@@ -1,6 +1,7 @@
 // hg_api.cu -- the C ABI of include/hg.h: context, device buffers, the
 // explicit calls of one block step and the graph-captured device-resident
 // stepping loop.
+#include <cuda.h>
 #include <cuda_runtime.h>
 #include <math.h>
 #include <nvtx3/nvToolsExt.h>
@@ -157,17 +158,48 @@ bool is_device_ptr(const void *p)
     return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
-// Plain memory of the context's GPU, aligned for T: kernels may write it.
-template <class T>
-bool is_own_memory(const hg_ctx *c, const T *p)
-{
-    cudaPointerAttributes a;
-    if (!p || ((uintptr_t)p & (sizeof(T) - 1)) != 0) return false;
-    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
+// An allocation of plain memory on the context's GPU.
+struct Range {
+    CUdeviceptr base = 0;
+    size_t size = 0;
+    bool holds(CUdeviceptr at, size_t bytes) const
+    {
+        return at >= base && at - base <= size && bytes <= size - (at - base);
     }
-    return a.type == cudaMemoryTypeDevice && a.device == c->device;
+};
+
+// Plain memory of the context's GPU, aligned for T, and [p, p + count) inside its
+// allocation: kernels may write it.  (Anything else gets a copy.)  last: the allocation
+// found before in this call, often the same one.
+template <class T>
+bool is_own_memory(const hg_ctx *c, const T *p, int64_t count, Range &last)
+{
+    typedef CUresult (*QueryFn)(unsigned, CUpointer_attribute *, void **, CUdeviceptr);
+    static const QueryFn query = [] {
+        void *f = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &f, 12000, cudaEnableDefault, &q) != cudaSuccess ||
+            q != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            f = nullptr;
+        }
+        return reinterpret_cast<QueryFn>(f);
+    }();
+    if (!p || ((uintptr_t)p & (sizeof(T) - 1)) != 0 || !query) return false;
+    const CUdeviceptr at = (CUdeviceptr)(uintptr_t)p;
+    const size_t bytes = (size_t)count * sizeof(T);
+    if (last.holds(at, bytes)) return true;
+    unsigned type = 0, managed = 0;
+    int device = -1;
+    Range r;
+    CUpointer_attribute what[] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_IS_MANAGED,
+                                  CU_POINTER_ATTRIBUTE_DEVICE_ORDINAL, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR,
+                                  CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+    void *to[] = {&type, &managed, &device, &r.base, &r.size};
+    if (query(5, what, to, at) != CUDA_SUCCESS || type != CU_MEMORYTYPE_DEVICE || managed || device != c->device)
+        return false;
+    last = r;
+    return r.holds(at, bytes);
 }
 
 template <class T>
@@ -938,7 +970,8 @@ int hg_next_block(hg_ctx *c, double *t_next, int32_t *idx, int64_t cap, int64_t 
     if (!c) return HG_EINVAL;
     if (const int rb = sync_bound(c)) return rb;
     // A device array that holds any block takes the list from the kernels.
-    const bool direct = cap >= c->n && is_own_memory(c, idx);
+    Range range;
+    const bool direct = cap >= c->n && is_own_memory(c, idx, c->n, range);
     HG_CUDA(c, launch_next_block(c->st, c->n, c->nb_part, c->nb_cnt, c->nb_off, c->d_idx, direct ? idx : nullptr,
                                  c->d_sc, c->stream));
     c->kernels += next_block_kernels(c->n);
@@ -1003,8 +1036,9 @@ int hg_evaluate(hg_ctx *c, const int32_t *idx, int64_t m, double *acc, double *j
         // (then copied one after the other).
         double *outs[3] = {acc, jerk, snap};
         EvalOut direct;
+        Range range;
         for (int k = 0; k < 3; ++k)
-            if (is_own_memory(c, outs[k])) direct.p[k] = outs[k];
+            if (is_own_memory(c, outs[k], 3 * m, range)) direct.p[k] = outs[k];
         for (int k = 0; k < 3; ++k)
             for (int j = 0; j < k; ++j)
                 if (outs[j] && outs[k] && outs[k] < outs[j] + 3 * m && outs[j] < outs[k] + 3 * m) direct = EvalOut{};
