@@ -453,8 +453,10 @@ int ensure_graphs(hg_ctx *c)
         c->kernels += 1;
         c->plan_tab_valid = true;
     }
-    if (!c->g_one[c->par]) rc = capture(c, 1, c->par, &c->g_one[c->par], c->ev_one);
-    if (rc == HG_OK && !c->g_many[c->par])
+    // Both lengths at the first call; those of the other entry when they are replayed
+    // (single steps in turn need one of them).
+    if (!c->g_one[0] && !c->g_one[1]) rc = capture(c, 1, c->par, &c->g_one[c->par], c->ev_one);
+    if (rc == HG_OK && !c->g_many[0] && !c->g_many[1])
         rc = capture(c, c->opts.graph_steps, c->par, &c->g_many[c->par], c->ev_many);
     return rc;
 }
@@ -464,7 +466,7 @@ int replay(hg_ctx *c, bool many)
 {
     const int steps = many ? c->opts.graph_steps : 1;
     cudaGraphExec_t &g = many ? c->g_many[c->par] : c->g_one[c->par];
-    if (!g) {   // an odd number of steps came before
+    if (!g) {   // the other entry: an odd number of steps came before
         const int rc = capture(c, steps, c->par, &g, many ? c->ev_many : c->ev_one);
         if (rc) return rc;
     }
