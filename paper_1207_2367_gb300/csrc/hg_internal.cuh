@@ -26,7 +26,7 @@ struct DevScalars {
     // selection can clear what its correction and the next selection will write.
     unsigned long long slot[2];   // active-list entries taken by the fused selection
     int64_t tnext_bits[2];        // bit pattern of min_i tend_i (next-block pass 1, or a correction)
-    uint32_t arrive[4];    // CTAs done in next-block passes 1 and 2 (the last one resets it); two spare
+    uint32_t arrive[2];    // CTAs done in next-block passes 1 and 2 (the last one resets it)
 };
 
 enum : int32_t { ERR_TIMEOUT = 1, ERR_BADIDX = 2, ERR_STATE = 4, ERR_VALUE = 8, ERR_BOUNDS = 16 };

@@ -10,7 +10,6 @@
 #include <stdint.h>
 
 #include "hg_kernels.cuh"
-#include "hg_plan_dev.cuh"
 
 namespace hg {
 namespace {
