@@ -127,8 +127,9 @@ struct FaultFromEnv {
 } g_fault_from_env;
 
 // Largest system whose graph steps read their plans from a table of all block sizes
-// (48 B each); beyond, where a step's prediction alone takes 35 us and more, a kernel
-// (2 us) scores the candidates of each step's block.
+// (48 B each: 50 MB at 2^20), made at the first graph step in 0.12 ms for 65536 particles
+// and 1.8 ms for 2^20.  Beyond, a kernel scores the candidates of each step's block: 5 us a
+// step (measured at 16385 to 2^20), which the table has saved after 25 and 350 steps.
 constexpr int64_t kPlanTable = (int64_t)1 << 20;
 
 constexpr cudaError_t kInjected = cudaErrorUnknown;

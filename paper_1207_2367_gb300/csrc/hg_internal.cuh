@@ -167,37 +167,59 @@ __host__ __device__ inline int64_t div_ceil(int64_t a, int64_t b)
     return (a + b - 1) / b;
 }
 
+// What a candidate is whatever the block size; wave_one, wave: its cost per wave of work
+// items when one wave holds them all, and when there are several.
+struct PlanShape {
+    int64_t tps, b, wave_one, wave;
+    int tpi, ti, v, grid;
+};
+__host__ __device__ inline bool plan_shape(const PlanParams &q, int c, PlanShape &s)
+{
+    s.v = c / kPlanCandidates;
+    if (c < 0 || s.v >= q.variants) return false;
+    c -= s.v * kPlanCandidates;
+    s.grid = s.v ? q.grid1 : q.grid;
+    s.tpi = 1 << (c / 32);
+    if (s.tpi > kMaxTPI || (q.tpi_force > 0 && s.tpi != q.tpi_force)) return false;
+    s.tps = plan_tps(c % 32);
+    if (q.b_force > 0) {
+        if (c % 32 != 0) return false;
+        const int64_t b = q.b_force < q.ntiles ? q.b_force : q.ntiles;
+        s.tps = div_ceil(q.ntiles, b);
+    }
+    if (s.tps > q.ntiles) return false;
+    s.b = div_ceil(q.ntiles, s.tps);
+    s.ti = kEvalThreads / s.tpi * (s.v ? q.ipt1 : q.i_per_thread);
+    s.wave_one = s.tps * ((q.tj / s.tpi) * (s.v ? q.weight1_one : 100) + q.c_tile * 100) + q.c_item * 100;
+    s.wave = s.v ? s.tps * ((q.tj / s.tpi) * q.weight1 + q.c_tile * 100) + q.c_item * 100 : s.wave_one;
+    return true;
+}
+
+// Modelled cost of a block of m > 0 (-1: its partial sums do not fit the buffer): waves *
+// (tiles per item * (TJ / tpi + c_tile) + c_item), integers only so that host and device
+// choose the same plan.
+__host__ __device__ inline int64_t plan_cost(int64_t m, const PlanParams &q, const PlanShape &s)
+{
+    if (s.b * m > q.pcap && s.b > 1) return -1;
+    const int64_t waves = div_ceil(div_ceil(m, s.ti) * s.b, s.grid);
+    return waves * (waves > 1 ? s.wave : s.wave_one);
+}
+
 // Fill p for candidate c and return its modelled cost (-1: not admissible).
-// cost = waves * (tiles per item * (TJ / tpi + c_tile) + c_item), integers only
-// so that host and device choose the same plan.
 __host__ __device__ inline int64_t plan_candidate(int64_t m, const PlanParams &q, int c, Plan &p)
 {
-    const int v = c / kPlanCandidates;
-    if (c < 0 || v >= q.variants) return -1;
-    c -= v * kPlanCandidates;
-    const int ipt = v ? q.ipt1 : q.i_per_thread, grid = v ? q.grid1 : q.grid;
-    const int tpi = 1 << (c / 32);
-    if (tpi > kMaxTPI || (q.tpi_force > 0 && tpi != q.tpi_force)) return -1;
-    int64_t tps = plan_tps(c % 32);
-    if (q.b_force > 0) {
-        if (c % 32 != 0) return -1;
-        const int64_t b = q.b_force < q.ntiles ? q.b_force : q.ntiles;
-        tps = div_ceil(q.ntiles, b);
-    }
-    if (tps > q.ntiles) return -1;
-    const int64_t b = div_ceil(q.ntiles, tps);
-    const int64_t mm = m > 0 ? m : 1;
-    if (b * mm > q.pcap && b > 1) return -1;
-    p.tpi = tpi;
-    p.ti = kEvalThreads / tpi * ipt;
-    p.n_itiles = div_ceil(mm, p.ti);
-    p.tiles_per_split = tps;
-    p.b = (int)b;
-    p.variant = v;
-    p.n_items = p.n_itiles * b;
-    const int64_t waves = div_ceil(p.n_items, grid);
-    const int64_t w = v == 0 ? 100 : (waves > 1 ? q.weight1 : q.weight1_one);
-    return waves * (tps * ((q.tj / tpi) * w + q.c_tile * 100) + q.c_item * 100);
+    PlanShape s;
+    if (!plan_shape(q, c, s)) return -1;
+    const int64_t mm = m > 0 ? m : 1, cost = plan_cost(mm, q, s);
+    if (cost < 0) return -1;
+    p.tpi = s.tpi;
+    p.ti = s.ti;
+    p.n_itiles = div_ceil(mm, s.ti);
+    p.tiles_per_split = s.tps;
+    p.b = (int)s.b;
+    p.variant = s.v;
+    p.n_items = p.n_itiles * s.b;
+    return cost;
 }
 
 __host__ __device__ inline int plan_total(const PlanParams &q) { return q.variants * kPlanCandidates; }
