@@ -180,7 +180,9 @@ __global__ void __launch_bounds__(kNBThreads) k_nb_scatter(const double *tend, i
 // The three passes of a small system in one CTA: up to kSmallPer end times a thread,
 // read once; their minimum, then the ascending list from the ballots of every row of
 // 1024 particles.  Fixed latencies (three launches, two arrival counts) made the
-// passes 4.5 + 4.3 + 5.2 us at N = 1024; this is 3.8 us.
+// passes 4.5 + 4.3 + 5.2 us at N = 1024; this is 3.8 us.  The whole of hg_next_block, three
+// passes and this one: 28.3 and 16.6 us for 64 particles, 28.6 and 16.6 for 1024, 31.6 and
+// 16.9 for 4096, 33.1 and 17.3 for 8192, the most that kSmallPer registers a thread hold.
 constexpr int kSmallThreads = 1024, kSmallPer = 8;
 
 __global__ void __launch_bounds__(kSmallThreads) k_nb_small(const double *tend, int64_t n, int32_t *idx, int32_t *out,
