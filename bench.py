@@ -56,7 +56,7 @@ NUM_SMS = 152
 # (N, masses, precision, warm-up steps, timed steps); valid only while that
 # kernel is unchanged (None: not captured for the current kernel).
 EVAL_TRAFFIC = {
-    # the default line with the driver's --steps 20 --warmup 5: 20 launches, 1.962e12 B in 27.4 s of kernel time
+    # the default line with --steps 20 --warmup 5: 20 launches, 1.962e12 B in 27.4 s of kernel time
     # (72 GB/s); the i-tiles re-read the 436 MB of records from DRAM as they drift apart along them
     (8388608, "salpeter", "mixed", 5, 20): 9.8116e10,
 }
@@ -329,8 +329,8 @@ def roofline(hg, inter, prof, mixed, mhz, kind, traffic=None, measured=None):
            "flops_per_interaction_rsqrt_as_4": flops + 4,
            "paper_flops_per_interaction": PAPER_FLOPS,
            "peak_note": ((f"FP32 FMA pipe: {NUM_SMS} SMs x 128 lanes x 2 flops" if mixed else
-                          f"FP64 pipe: {NUM_SMS} SMs x 2 DFMA x 2 flops; all but the differences of a pair run as "
-                          f"64-bit fixed point on the integer pipes, so the share may exceed 1,")
+                          f"FP64 pipe: {NUM_SMS} SMs x 2 DFMA x 2 flops; the differences, w and the sums of a pair "
+                          f"run there, the rest of it on the integer pipes, so the share may exceed 1,")
                          + f" x {mhz:.0f} MHz ({kind} max clock)"),
            "eval_share_of_step": eval_s / (sum(prof["ms"].values()) / 1e3) if prof["ms"] else None}
     if measured:
@@ -897,7 +897,7 @@ def run_batch(a):
 
 
 # ----------------------------------------------------------------------------
-# Further configurations (one JSON line each; not the driver's default line).
+# Further configurations (one JSON line each; not the default line).
 # ----------------------------------------------------------------------------
 def _device_state(hg, ctx, n):
     import torch

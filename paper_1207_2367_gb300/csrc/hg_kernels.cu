@@ -508,7 +508,7 @@ __global__ void __launch_bounds__(kPotThreads) k_potential_mixed(const double *x
 // are split once per block and tile.  N = 65536: 106 ms with FP64 instructions
 // throughout (16 a pair, 64 cycles each per warp) and every pair from both sides,
 // 37.1 ms in fixed point, now 16.9 ms; bound by the integer pipes' issue and the
-// three FP64 subtractions (192 of ~330 cycles per warp and pair).
+// three FP64 subtractions (192 of ~295 cycles per warp and pair at 1.92 GHz).
 __global__ void __launch_bounds__(kPotThreads) k_potential_fp64(const double *xe, const double *mass, int64_t n,
                                                                  double eps2, double *phi_part)
 {
